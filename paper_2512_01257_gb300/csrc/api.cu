@@ -7,6 +7,7 @@
 // graphs of `chunk` steps and replayed until the device reports that every
 // system has converged.
 #include <algorithm>
+#include <array>
 #include <atomic>
 #include <cmath>
 #include <cstdio>
@@ -1042,6 +1043,451 @@ static void filter_ms_dev(Handle* h, const rafeast_params& prm, const double* Qd
 }
 
 // ---------------------------------------------------------------------------
+// real Lanczos form of the multi-shift filter (lanczos.cuh): the default. Same
+// Q~ as filter_ms_dev in exact arithmetic.
+// ---------------------------------------------------------------------------
+template <typename T>
+struct LzProblem {
+  LzArgs<T> a;
+  const double* fin = nullptr;  // device [m0]: per-column constant of the correction form
+  int m0 = 0;
+};
+
+// ---- the ring of Lanczos vectors (Handle::lz_slabs) ---------------------------
+// Slots are allocated as a solve needs them, up to a share of the device's
+// memory (LZ_RING_SHARE); a solve with more steps than slots folds full rings
+// into its directions. A slab is about a gigabyte or the whole of 32 slots.
+constexpr size_t LZ_RING_SHARE = 16;  // a sixteenth of the device's memory
+static void lz_free(Handle* h) {
+  for (void* p : h->lz_slabs) cudaFree(p);
+  h->lz_slabs.clear();
+  h->lz_stride = 0;
+  for (int slot : {S_LZP, S_LZC})
+    if ((int)h->bufs.size() > slot && h->bufs[slot].p) {
+      cudaFree(h->bufs[slot].p);
+      h->bufs[slot] = DevBuf();
+    }
+}
+// slots of `stride` bytes: `least` of them, or it throws, and `want` if they
+// can be had within `budget` bytes; returns the slots there are
+static int lz_grow(Handle* h, int64_t stride, int sl, int64_t least, int64_t want,
+                   size_t budget) {
+  if (h->lz_stride != stride || h->lz_sl != sl) {
+    for (void* p : h->lz_slabs) RF_CUDA(cudaFree(p));
+    h->lz_slabs.clear();
+    h->lz_stride = stride;
+    h->lz_sl = sl;
+  }
+  const size_t bytes = (size_t)stride * sl;
+  while ((int64_t)h->lz_slabs.size() * sl < want && h->lz_slabs.size() < (size_t)LZ_SLABS) {
+    const bool must = (int64_t)h->lz_slabs.size() * sl < least;
+    if (!must && (h->lz_slabs.size() + 1) * bytes > budget) break;
+    void* p = nullptr;
+    const cudaError_t e = cudaMalloc(&p, bytes);
+    if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
+      if (!must) break;
+      throw Err{RAFEAST_ERR_OUT_OF_MEMORY};
+    }
+    RF_CUDA(e);
+    h->lz_slabs.push_back(p);
+  }
+  return (int)std::min<int64_t>((int64_t)h->lz_slabs.size() * sl, 1 << 20);
+}
+
+// the slab table and the slot count to the device (no step in flight)
+template <typename T>
+static void lz_ring_upload(Handle* h, const LzArgs<T>& a, cudaStream_t st) {
+  LzDyn d;
+  memset(&d, 0, sizeof(d));
+  for (size_t t = 0; t < h->lz_slabs.size(); ++t) d.slab[t] = (char*)h->lz_slabs[t];
+  d.cap = (int)h->lz_slabs.size() * a.sl;
+  RF_CUDA(cudaMemcpyAsync(a.dyn, &d, offsetof(LzDyn, k), cudaMemcpyHostToDevice, st));
+}
+
+// the steps [k0, k1) of a problem into D (and, unless the solve is over, into
+// its directions)
+template <typename T>
+static void lz_collapse(Handle* h, LzArgs<T> a, int k0, int k1, bool last, cudaStream_t st) {
+  if (k1 <= k0) return;
+  const bool dirs = !last || k0 > 0;
+  const size_t n_cc = (size_t)(k1 - k0) * a.ld;
+  a.cc = (T*)scratch(h, S_LZC, sizeof(T) * n_cc * (dirs ? 1 + 2 * (size_t)a.nc : 1));
+  a.bb = a.cc + n_cc;
+  if (dirs) a.p = (T*)scratch(h, S_LZP, (size_t)2 * a.nc * h->n * a.ld * sizeof(T));
+  launch_lz_collapse<T>(a, k0, k1, last, h->num_sms, st);
+  h->launches += dirs ? 1 + (a.nc + 3) / 4 : 2;
+}
+
+// steps per graph replay (even)
+static int lz_replay_steps(const Handle* h, bool tight) {
+  if (tight) return 2;
+  return std::min(62, std::max(2, h->opt_chunk + (h->opt_chunk & 1)));
+}
+
+// quadrature, coefficient upload and state init of one problem on stream st
+// (one launch). ctl_dev replaces the handle's own control block (batches).
+template <typename T>
+static LzProblem<T> lz_setup(Handle* h, const rafeast_params& prm, const double* Qd,
+                             const double* AQd, const double* theta_d,
+                             const std::vector<double>& theta, int m0, int ldq, CocgCtl* ctl_dev,
+                             bool profile, bool tight, cudaStream_t st) {
+  const bool fp64 = sizeof(T) == 8;
+  std::vector<double> zr, zi, wr, wi;
+  quadrature_nodes(prm.lmin, prm.lmax, prm.nc, prm.ellipse_ratio, zr, zi, wr, wi);
+  shard_nodes(h, zr, zi, wr, wi);
+  const int nc = (int)zr.size();
+  const bool corr = prm.solve_form == RAFEAST_FORM_CORRECTION;
+  const int ld = (m0 + 3) & ~3, V = 16 / (int)sizeof(T), nq = ld / V;
+  // one upload: nodes, coefficients, the correction form's column constants
+  const size_t n_z = nc, n_coef = (size_t)ld * nc;
+  std::vector<double> up(2 * (n_z + n_coef) + m0, 0.0);
+  double *hz = up.data(), *hc = hz + 2 * n_z, *hf = hc + 2 * n_coef;
+  for (int j = 0; j < nc; ++j) {
+    hz[2 * j] = zr[j] - h->shift;
+    hz[2 * j + 1] = zi[j];
+  }
+  for (int i = 0; i < m0; ++i)
+    for (int j = 0; j < nc; ++j) {
+      double re = wr[j], im = wi[j];
+      if (corr) {
+        const double dr = zr[j] - theta[i], di = zi[j], den = dr * dr + di * di;
+        re = (wr[j] * dr + wi[j] * di) / den;
+        im = (wi[j] * dr - wr[j] * di) / den;
+        hf[i] += re;
+      }
+      hc[2 * ((size_t)i * nc + j)] = re;
+      hc[2 * ((size_t)i * nc + j) + 1] = im;
+    }
+  LzArgs<T> a;
+  memset(&a, 0, sizeof(a));
+  a.n = h->n;
+  a.rowptr = h->rowptr;
+  a.colidx = h->colidx;
+  a.val = fp64 ? (const T*)h->val64 : (const T*)h->val32;
+  if (h->lcolidx && h->opt_values_free == 0) {
+    a.lrowptr = h->lrowptr;
+    a.lcolidx = h->lcolidx;
+  }
+  a.ld = ld;
+  a.nq = nq;
+  a.nc = nc;
+  const int64_t block = h->n * (int64_t)ld * sizeof(T);
+  a.uoff = (block + 255) & ~(int64_t)255;
+  a.stride = (a.uoff + (int64_t)sizeof(double2) * 2 * ld * nc + 255) & ~(int64_t)255;
+  // 32 slots a slab, fewer when that is over a gigabyte; 4 when memory is short
+  a.sl = tight ? 4 : (int)std::max<int64_t>(8, std::min<int64_t>(LZ_SL, ((int64_t)1 << 30) / a.stride));
+  int blocks = 1;
+  choose_shape(nq, 2, fp64, h->opt_lanes, a.lanes, a.cpl, blocks,
+               h->opt_cpl > 0 ? std::min(h->opt_cpl, 4) : 2);
+  a.w = (T*)scratch(h, S_STATE, block);
+  a.dacc = (T*)scratch(h, S_DACC, block);
+  const int least = lz_replay_steps(h, tight) + 2;  // a replay's slots and u_{k0-1}
+  lz_grow(h, a.stride, a.sl, least, least, 0);
+  if (tight) scratch(h, S_LZP, (size_t)2 * nc * block);
+  size_t off = 0;
+  auto carve = [&](size_t bytes) {
+    off = (off + 255) & ~(size_t)255;
+    size_t o = off;
+    off += bytes;
+    return o;
+  };
+  const size_t o_up = carve(sizeof(double) * up.size());
+  const size_t o_acc = carve(sizeof(double) * 2 * ld);
+  const size_t o_col = carve(sizeof(LzCol) * ld);
+  const size_t o_sh = carve(sizeof(LzShift) * ld * nc);
+  const size_t o_cf = carve(sizeof(LzCoef<T>) * ld);
+  const size_t o_qact = carve(sizeof(int) * nq);
+  const size_t o_head = carve(sizeof(T) * 4 * (size_t)ld * nc);
+  const size_t o_dyn = carve(sizeof(LzDyn));
+  const size_t o_flag = carve(sizeof(int) * ld * nc);
+  const size_t o_ctl = carve(sizeof(CocgCtl));
+  const size_t o_hist = carve(sizeof(int) * ((size_t)prm.max_inner + 2));
+  const size_t o_rhist = carve(sizeof(double) * ((size_t)prm.max_inner + 2));
+  char* sc = (char*)scratch(h, S_SCAL, off + 256);
+  RF_CUDA(cudaMemcpyAsync(sc + o_up, up.data(), sizeof(double) * up.size(),
+                          cudaMemcpyHostToDevice, st));
+  a.z = (const double2*)(sc + o_up);
+  a.coef = a.z + n_z;
+  a.acc = (double*)(sc + o_acc);
+  a.col = (LzCol*)(sc + o_col);
+  a.sh = (LzShift*)(sc + o_sh);
+  a.cf = (LzCoef<T>*)(sc + o_cf);
+  a.qact = (int*)(sc + o_qact);
+  a.hd = (T*)(sc + o_head);
+  a.dyn = (LzDyn*)(sc + o_dyn);
+  a.pflag = (int*)(sc + o_flag);
+  a.ctl = ctl_dev ? ctl_dev : (CocgCtl*)(sc + o_ctl);
+  a.hist = profile ? (int*)(sc + o_hist) : nullptr;
+  a.rhist = profile ? (double*)(sc + o_rhist) : nullptr;
+  a.tol2 = prm.solve_tol * prm.solve_tol;
+  a.max_inner = prm.max_inner;
+  lz_ring_upload(h, a, st);
+  launch_lz_init<T>(a, Qd, AQd, theta_d, ldq, m0, prm.solve_form, h->num_sms, st);
+  h->launches += 1;
+  LzProblem<T> P;
+  P.a = a;
+  P.fin = (const double*)(sc + o_up) + 2 * (n_z + n_coef);
+  P.m0 = m0;
+  return P;
+}
+
+// algorithmic bytes of a step with `cols` active columns: the product reads A
+// and u and writes w; the update reads u, w, u_{k-1} and writes u_{k+1}
+static double lz_dots_bytes(const Handle* h, int cols, bool fp64, bool vf) {
+  const double sv = fp64 ? 8.0 : 4.0;
+  const double abytes = vf ? (double)h->nnz_off * 4.0 + 4.0 * (h->n + 1)
+                           : (double)h->nnz * (4.0 + sv) + 4.0 * (h->n + 1);
+  return abytes + 2.0 * sv * (double)h->n * cols;
+}
+static double lz_update_bytes(const Handle* h, int cols, int k, bool fp64) {
+  return (k == 0 ? 3.0 : 4.0) * (fp64 ? 8.0 : 4.0) * (double)h->n * cols;
+}
+
+template <typename T>
+static void lz_finish_filter(Handle* h, const LzProblem<T>& P, const double* Qd, int ldq,
+                             double* Qt, const CocgCtl& ctl, FilterStats& fs, cudaStream_t st) {
+  if (!ctl.done || ctl.timeout) throw Err{RAFEAST_ERR_TIMEOUT};
+  fs.iters_max = ctl.max_iters;
+  fs.iters_min = ctl.min_iters;
+  fs.breakdown = ctl.breakdown;
+  fs.capped = ctl.capped;
+  launch_combine<T>(Qd, ldq, P.a.dacc, P.a.ld, P.fin, h->n, P.m0, Qt, st);
+  h->launches += 1;
+  if (fs.breakdown) throw Err{RAFEAST_ERR_COCG_BREAKDOWN};
+}
+
+template <typename T>
+static void filter_lz_run(Handle* h, const rafeast_params& prm, const double* Qd,
+                          const double* AQd, const double* theta_d,
+                          const std::vector<double>& theta, int m0, int ldq, double* Qt,
+                          FilterStats& fs, bool tight) {
+  const bool fp64 = sizeof(T) == 8, prof = h->opt_profile != 0;
+  cudaStream_t st = h->stream;
+  LzProblem<T> P =
+      lz_setup<T>(h, prm, Qd, AQd, theta_d, theta, m0, ldq, nullptr, prof, tight, st);
+  LzArgs<T>& a = P.a;
+  const bool vf = a.lcolidx != nullptr;
+  const bool can_tile = !fp64 && h->ntiles > 0 && h->opt_tiled != 1 &&
+                        (vf ? h->llidx != nullptr : h->lidx != nullptr);
+  double* tpart = can_tile ? (double*)scratch(h, S_TPART, sizeof(double) * (size_t)h->num_sms *
+                                                              TILE_MAX_OCC * 16 * 10)
+                           : nullptr;
+  auto dots = [&](const LzArgs<T>& ad, int cb, int occ) {
+    if constexpr (std::is_same<T, float>::value) {
+      if (cb > 0) {
+        TileArgs tl;
+        tl.ntiles = h->ntiles;
+        tl.max_union = h->tile_max_union;
+        tl.trow = h->trow;
+        tl.uoff = h->uoff;
+        tl.ucol = h->ucol;
+        tl.uself = h->uself;
+        tl.lidx = vf ? h->llidx : h->lidx;
+        tl.cb = cb;
+        tl.ncb = (a.nq + cb - 1) / cb;
+        tl.part = tpart;
+        launch_lz_dots_tiled(ad, tl, h->num_sms, occ, st);
+        return;
+      }
+    }
+    launch_lz_dots<T>(ad, occ, h->num_sms, st);
+  };
+  // autotuner of the product's shape, once per handle, subspace width and
+  // precision: the candidates run on u_0 with nothing advancing (a.dry), timed
+  // back to back. Shapes change the work split, not the arithmetic of a row.
+  const int64_t key = ((int64_t)a.nq << 20) | (vf ? 8 : 0) | 4 | (fp64 ? 1 : 0);
+  int cb = 0, occ = 0;
+  bool have = false;
+  for (auto& kv : h->tuned)
+    if (kv.first == key) {
+      a.lanes = kv.second.dl;
+      a.cpl = kv.second.dc;
+      occ = kv.second.dm;
+      cb = can_tile ? kv.second.dt : 0;
+      have = h->opt_tiled != 2 || !can_tile || cb > 0;
+    }
+  const bool tune = h->opt_autotune && !h->opt_lanes && !h->opt_cpl;
+  if (!have && !tune && can_tile && h->opt_tiled == 2) cb = 8;
+  if (!have && tune) {
+    struct Cand {
+      int lanes, cpl, occ, cb;
+    };
+    std::vector<Cand> cand;
+    if (h->opt_tiled != 2 || !can_tile)
+      for (const auto& c : {std::array<int, 3>{32, 1, 0}, {32, 1, 3}, {16, 1, 0}, {16, 1, 3},
+                            {16, 2, 0}, {16, 2, 2}, {8, 1, 0}, {8, 2, 0}, {8, 2, 2}, {8, 3, 0},
+                            {8, 4, 0}, {4, 1, 0}, {4, 2, 0}, {4, 4, 0}}) {
+        const int w = c[0] * c[1], blocks = (a.nq + w - 1) / w;
+        if ((double)a.nq / (blocks * w) >= 0.5 || (c[0] == 4 && c[1] == 1))
+          cand.push_back({c[0], c[1], c[2], 0});
+      }
+    if (can_tile)
+      for (const auto& c : {std::array<int, 2>{8, 0}, {4, 0}, {5, 0}, {10, 0}, {8, 2}})
+        if (c[0] == 4 || (double)a.nq / ((a.nq + c[0] - 1) / c[0] * c[0]) >= 0.75 ||
+            (c[0] == 8 && a.nq > 4))
+          cand.push_back({a.lanes, a.cpl, c[1], c[0]});
+    const int runs = 2;
+    std::vector<cudaEvent_t> evs(cand.size() * runs + 1);
+    for (auto& e : evs) RF_CUDA(cudaEventCreate(&e));
+    LzArgs<T> t = a;
+    t.dry = 1;
+    for (size_t ci = 0; ci < cand.size(); ++ci) {
+      t.lanes = cand[ci].lanes;
+      t.cpl = cand[ci].cpl;
+      for (int r = 0; r < runs; ++r) {
+        RF_CUDA(cudaEventRecord(evs[ci * runs + r], st));
+        dots(t, cand[ci].cb, cand[ci].occ);
+      }
+    }
+    RF_CUDA(cudaEventRecord(evs.back(), st));
+    RF_CUDA(cudaStreamSynchronize(st));
+    h->launches += (int)cand.size() * runs;
+    float best = 1e30f;
+    for (size_t ci = 0; ci < cand.size(); ++ci) {
+      float ms = 0.f;  // the second run: the first may have loaded the kernel
+      RF_CUDA(cudaEventElapsedTime(&ms, evs[ci * runs + runs - 1], evs[ci * runs + runs]));
+      // a tiled product adds its sums in a fixed order (solves repeat to the
+      // last bit): it is kept unless the gathers are more than 5% faster
+      if (cand[ci].cb) ms /= 1.05f;
+      if (ms < best) {
+        best = ms;
+        a.lanes = cand[ci].lanes;
+        a.cpl = cand[ci].cpl;
+        occ = cand[ci].occ;
+        cb = cand[ci].cb;
+      }
+    }
+    for (auto& e : evs) RF_CUDA(cudaEventDestroy(e));
+    Handle::Shape shp{a.lanes, a.cpl, 0, 0};
+    shp.dm = occ;
+    shp.dt = cb;
+    h->tuned.push_back(std::make_pair(key, shp));
+  }
+  if (can_tile && h->opt_tiled == 2 && h->opt_tile_cb > 0) {
+    cb = h->opt_tile_cb;  // forced block width (tests)
+    occ = 0;
+  }
+  h->prof[6] = cb ? 1000000 + cb * 100 + occ : occ * 10000 + a.lanes * 100 + a.cpl;
+  h->prof[7] = a.sl;
+  // a graph of `steps` steps, replayed until done; the ring grows before a
+  // replay that needs more slots, or is folded into D when it may not
+  const int steps = lz_replay_steps(h, tight);
+  std::vector<cudaEvent_t> evs;
+  if (prof) {
+    evs.resize(2 * steps + 1);
+    for (auto& e : evs) RF_CUDA(cudaEventCreate(&e));
+  }
+  struct ExecGuard {  // the graph goes with the call, whichever way it ends
+    cudaGraphExec_t exec = nullptr;
+    ~ExecGuard() {
+      if (exec) cudaGraphExecDestroy(exec);
+    }
+  } guard;
+  cudaGraphExec_t& exec = guard.exec;
+  cudaGraph_t graph = nullptr;
+  RF_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+  g_capturing = true;
+  try {
+    for (int it = 0; it < steps; ++it) {
+      if (prof) RF_CUDA(cudaEventRecordWithFlags(evs[2 * it], st, cudaEventRecordExternal));
+      dots(a, cb, occ);
+      if (prof) RF_CUDA(cudaEventRecordWithFlags(evs[2 * it + 1], st, cudaEventRecordExternal));
+      launch_lz_update<T>(a, h->num_sms, st);
+    }
+    if (prof) RF_CUDA(cudaEventRecordWithFlags(evs[2 * steps], st, cudaEventRecordExternal));
+  } catch (...) {
+    g_capturing = false;
+    cudaStreamEndCapture(st, &graph);
+    if (graph) cudaGraphDestroy(graph);
+    throw;
+  }
+  g_capturing = false;
+  RF_CUDA(cudaStreamEndCapture(st, &graph));
+  RF_CUDA(cudaGraphInstantiate(&exec, graph, 0));
+  RF_CUDA(cudaGraphDestroy(graph));
+  std::vector<float> tk;  // per step: product ms, update ms (profiling)
+  CocgCtl ctl;
+  memset(&ctl, 0, sizeof(ctl));
+  if (!h->mem_total) {
+    size_t mem_free = 0;
+    RF_CUDA(cudaMemGetInfo(&mem_free, &h->mem_total));
+  }
+  const size_t budget = tight ? 0 : h->mem_total / LZ_RING_SHARE;
+  int k0 = 0, cap = (int)h->lz_slabs.size() * a.sl;
+  bool wrapped = false;
+  const int max_replays = (prm.max_inner + 2) / steps + 2;
+  for (int r = 0; r < max_replays && !ctl.done; ++r) {
+    const int k = ctl.iter;
+    if (k - k0 + steps + 1 > cap && !wrapped) {
+      const int64_t want = (int64_t)k + steps + 1;
+      const int got = lz_grow(h, a.stride, a.sl, 0, want, budget);
+      if (got != cap) {
+        cap = got;
+        lz_ring_upload(h, a, st);
+      }
+    }
+    if (k - k0 + steps + 1 > cap) {
+      wrapped = true;  // (step k uses slot k mod cap: cap stays from here on)
+      lz_collapse<T>(h, a, k0, k, false, st);
+      k0 = k;
+    }
+    RF_CUDA(cudaGraphLaunch(exec, st));
+    RF_CUDA(cudaMemcpyAsync(&ctl, a.ctl, sizeof(ctl), cudaMemcpyDeviceToHost, st));
+    RF_CUDA(cudaStreamSynchronize(st));
+    if (prof)
+      for (int it = 0; it < 2 * steps; ++it) {
+        float ms = 0.f;
+        RF_CUDA(cudaEventElapsedTime(&ms, evs[it], evs[it + 1]));
+        tk.push_back(ms);
+      }
+    h->launches += 2 * steps;
+    h->spmm_launches += steps;
+  }
+  lz_collapse<T>(h, a, k0, ctl.iter, true, st);
+  for (auto& e : evs) RF_CUDA(cudaEventDestroy(e));
+  if (prof && ctl.done) {
+    const int iters = std::min(ctl.iter, prm.max_inner + 1);
+    std::vector<int> hist(iters, 0);
+    RF_CUDA(cudaMemcpy(hist.data(), a.hist, sizeof(int) * iters, cudaMemcpyDeviceToHost));
+    h->last_hist = hist;
+    h->last_rhist.assign(iters, 0.0);
+    RF_CUDA(cudaMemcpy(h->last_rhist.data(), a.rhist, sizeof(double) * iters,
+                       cudaMemcpyDeviceToHost));
+    h->last_tk.assign(tk.begin(), tk.begin() + std::min<size_t>(tk.size(), 2 * (size_t)iters));
+    for (int k = 0; k < iters && 2 * k + 1 < (int)tk.size(); ++k) {
+      h->prof[0] += 1;
+      h->prof[1] += tk[2 * k];
+      h->prof[2] += lz_dots_bytes(h, k == 0 ? m0 : hist[k - 1], fp64, vf);
+      if (hist[k] > 0) {
+        h->prof[3] += 1;
+        h->prof[4] += tk[2 * k + 1];
+        h->prof[5] += lz_update_bytes(h, hist[k], k, fp64);
+      }
+    }
+  }
+  lz_finish_filter<T>(h, P, Qd, ldq, Qt, ctl, fs, st);
+}
+
+// (when memory runs out, once more with the smallest ring, whose state is no
+// larger than that of the COCG kernels)
+template <typename T>
+static void filter_lz_dev(Handle* h, const rafeast_params& prm, const double* Qd,
+                          const double* AQd, const double* theta_d,
+                          const std::vector<double>& theta, int m0, int ldq, double* Qt,
+                          FilterStats& fs) {
+  try {
+    filter_lz_run<T>(h, prm, Qd, AQd, theta_d, theta, m0, ldq, Qt, fs, false);
+  } catch (const Err& e) {
+    if (e.code != RAFEAST_ERR_OUT_OF_MEMORY) throw;
+    RF_CUDA(cudaStreamSynchronize(h->stream));
+    lz_free(h);
+    clear_last_error();
+    filter_lz_run<T>(h, prm, Qd, AQd, theta_d, theta, m0, ldq, Qt, fs, true);
+  }
+}
+
+// ---------------------------------------------------------------------------
 // batched multi-shift filter: the COCG steps of every problem of a batch run
 // in grouped launches (one dot and one update launch per step for all
 // problems, kernels_batched.cu) captured as one CUDA graph of `chunk` steps on
@@ -1332,11 +1778,14 @@ static void run_filter(Handle* h, const rafeast_params& prm, const double* Qd, c
                        double* Qt, FilterStats& fs) {
   // one COCG per shift is compiled for up to 8 shifts: more go multi-shift
   const bool ms = (h->opt_solver == 1 && h->opt_kernel != 2) || prm.nc > 8;
+  const bool lz = ms && h->opt_update == 0 && h->opt_defer == 0;
   if (prm.precision == RAFEAST_FP64) {
-    if (ms) filter_ms_dev<double>(h, prm, Qd, AQd, theta_d, theta, m0, ldq, Qt, fs);
+    if (lz) filter_lz_dev<double>(h, prm, Qd, AQd, theta_d, theta, m0, ldq, Qt, fs);
+    else if (ms) filter_ms_dev<double>(h, prm, Qd, AQd, theta_d, theta, m0, ldq, Qt, fs);
     else filter_dev<double>(h, prm, Qd, AQd, theta_d, theta, m0, ldq, Qt, fs);
   } else {
-    if (ms) filter_ms_dev<float>(h, prm, Qd, AQd, theta_d, theta, m0, ldq, Qt, fs);
+    if (lz) filter_lz_dev<float>(h, prm, Qd, AQd, theta_d, theta, m0, ldq, Qt, fs);
+    else if (ms) filter_ms_dev<float>(h, prm, Qd, AQd, theta_d, theta, m0, ldq, Qt, fs);
     else filter_dev<float>(h, prm, Qd, AQd, theta_d, theta, m0, ldq, Qt, fs);
   }
 }
@@ -1886,6 +2335,7 @@ void rafeast_destroy(rafeast_t hh) {
   if (h->stream) cudaStreamSynchronize(h->stream);
   for (auto& b : h->bufs)
     if (b.p) cudaFree(b.p);
+  for (void* p : h->lz_slabs) cudaFree(p);
   void* ptrs[] = {h->rowptr, h->colidx, h->val64,   h->val32,   h->perm,  h->iperm,
                   h->Q,      h->AQ,     h->theta_d, h->lrowptr, h->lcolidx, h->trow,
                   h->uoff,   h->ucol,   h->uself,   h->lidx,    h->llidx};

@@ -161,6 +161,87 @@ template <typename T> struct CocgArgs {
   const int32_t* lcolidx;
 };
 
+// ---- real Lanczos form of the multi-shift solve (lanczos.cuh) ----------------
+constexpr int LZ_RUNS = 0x7fffffff;  // kstop of a column or node still iterating
+constexpr int LZ_SL = 32;            // most ring slots per slab
+constexpr int LZ_SLABS = 128;        // most slabs of a ring
+struct LzCol {  // per column
+  double rr, irr;  // u_k^T u_k and its reciprocal
+  double s, is;    // the scale that made u_k and its reciprocal
+  double sq;       // sqrt(||b||^2 rr) of the previous step
+  double bnorm2;   // ||b||_2^2
+  int bad;         // a scalar of this step is not finite
+  int kstop;       // step the column stopped at, LZ_RUNS before
+};
+struct LzShift {  // per (column, node)
+  double2 rho;   // residual r_k = rho_k u_k
+  double2 dinv;  // 1 / delta_{k-1}
+  int kstop;
+  int pad;
+};
+template <typename T> struct LzCoef {
+  T alpha, g, s, pad;
+};
+// the ring and where a step finds its slots (device; slab and cap are written
+// by the host while no step runs, the rest by the product's last CTA)
+struct LzDyn {
+  char* slab[LZ_SLABS];  // LzArgs::sl slots each
+  int cap;               // slots of the ring: step k uses slot k mod cap
+  int k;                 // step of the next product
+  char* du;              // its u_k
+  char* uu;              // the update's u_k, u_{k-1} (null at k = 0), u_{k+1}
+  char* up;
+  char* un;
+};
+template <typename T> struct LzArgs {
+  int64_t n;
+  const int32_t* rowptr;
+  const int32_t* colidx;
+  const T* val;
+  const int32_t* lrowptr;  // values-free gathers (lcolidx != null), as CocgArgs
+  const int32_t* lcolidx;
+  int ld;          // real values per row: columns rounded up to a multiple of 4
+  int nq;          // 16-byte chunks per row
+  int nc;          // nodes
+  int lanes, cpl;  // register-gather product: lanes per row, chunks per lane
+  int dry;         // 1: the product leaves every scalar as it is (timing runs)
+  LzDyn* dyn;
+  int sl;          // slots per slab
+  int64_t stride;  // bytes of a slot: u (n x ld), then t_k and w_j eta_k of every
+  int64_t uoff;    // (column, node), double2 pairs, at byte uoff
+  T* w;            // L u_k
+  T* dacc;         // quadrature sum, n x ld
+  T* p;            // directions: planes (re, im) of node j at p + (2 j) n ld, + n ld
+  const double2* z;     // [nc] nodes, the diagonal shift taken off
+  const double2* coef;  // [ld * nc] quadrature coefficients
+  double* acc;          // [2 ld] sums of the register-gather product (zeroed)
+  LzCol* col;           // [ld]
+  LzShift* sh;          // [ld * nc]
+  LzCoef<T>* cf;        // [ld]
+  int* qact;            // [nq] 1 while a column of the chunk is active
+  T* cc;                // collapsed coefficients of a chunk of steps (lz_comp_col)
+  T* bb;
+  T* hd;                // [4 nc ld]
+  int* pflag;           // [ld * nc] 1: p_j read, 2: p_j written
+  CocgCtl* ctl;
+  int* hist;
+  double* rhist;
+  double tol2;
+  int max_inner;
+};
+
+template <typename T>
+void launch_lz_init(const LzArgs<T>& a, const double* q, const double* aq, const double* theta,
+                    int ldq, int m, int form, int num_sms, cudaStream_t s);
+template <typename T>
+void launch_lz_dots(const LzArgs<T>& a, int occ, int num_sms, cudaStream_t s);
+template <typename T>
+void launch_lz_update(const LzArgs<T>& a, int num_sms, cudaStream_t s);
+// the steps [k0, k1) into D; last: the solve is over (no direction goes on)
+template <typename T>
+void launch_lz_collapse(const LzArgs<T>& a, int k0, int k1, bool last, int num_sms,
+                        cudaStream_t s);
+
 // ---- row tiles of the tiled sparse products (tiling.cpp, kernels_tiled.cu) ----
 // Tile t holds rows [trow[t], trow[t+1]); its union (the rows its nonzeros
 // name and its own rows, ascending) is ucol[uoff[t] .. uoff[t+1]); its first
@@ -199,6 +280,7 @@ struct DevBuf {
 struct Handle {
   int device = 0;
   int num_sms = 0;
+  size_t mem_total = 0;  // bytes of device memory
   int64_t n = 0, nnz = 0;
   cudaStream_t user_stream = nullptr;
   cudaStream_t stream = nullptr;  // internal, non-blocking
@@ -256,7 +338,8 @@ struct Handle {
   struct Shape {
     int dl, dc, ul, uc;
     int dm = 0, um = 0;  // forced CTAs per SM (0: default instance)
-    int dt = 0;          // tiled dot kernel: column pairs per block (0: register gathers)
+    int dt = 0;          // tiled dot kernel: column pairs (Lanczos form: chunks of
+                         // 4 columns) per block (0: register gathers)
   };
   std::vector<std::pair<int64_t, Shape>> tuned;
   int opt_profile = 0;
@@ -271,6 +354,11 @@ struct Handle {
   std::vector<float> last_tk;        // dot, update kernel milliseconds per step
   // scratch, grown on demand and kept
   std::vector<DevBuf> bufs;
+  // slabs of the Lanczos ring (lanczos.cuh), kept for the next solve while
+  // their slots have this many bytes
+  std::vector<void*> lz_slabs;
+  int64_t lz_stride = 0;
+  int lz_sl = 0;
   // launch accounting of the current call
   int launches = 0;
   int spmm_launches = 0;
@@ -283,7 +371,7 @@ void* scratch(Handle* h, int slot, size_t bytes);  // keep-alive buffer per slot
 void ensure_dyn_smem(const void* fn, size_t bytes);
 enum Slot {
   S_STATE = 0, S_DACC, S_QT, S_TMP1, S_TMP2, S_SCAL, S_GRAM, S_SMALL, S_OMEGA,
-  S_AQ2, S_IO1, S_IO2, S_BATCH, S_TPART, S_SHARD, S_COUNT
+  S_AQ2, S_IO1, S_IO2, S_BATCH, S_TPART, S_SHARD, S_LZ, S_LZP, S_LZC, S_COUNT
 };
 
 // ---- host math (hostmath.cpp) ------------------------------------------------
@@ -317,6 +405,9 @@ void tile_local_index(int64_t n, const int32_t* rowptr, const int32_t* colidx,
 // occ_cap: most CTAs per SM (0: as many as fit, at most TILE_MAX_OCC)
 void launch_ms_dots_tiled(const CocgArgs<float>& a, const TileArgs& tl, int buf, int num_sms,
                           int occ_cap, cudaStream_t s);
+// tiled product of the Lanczos form (float): tl.cb chunks of 4 columns per block
+void launch_lz_dots_tiled(const LzArgs<float>& a, const TileArgs& tl, int num_sms, int occ_cap,
+                          cudaStream_t s);
 
 // ---- kernel launchers (kernels_sparse.cu) --------------------------------------
 int nc_pad(int nc);  // shifts rounded up to a compiled NC (1, 2, 4, 8)

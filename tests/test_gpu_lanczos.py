@@ -1,0 +1,79 @@
+"""Real Lanczos form of the multi-shift filter (the default route) against the
+oracle's conjugate orthogonal CG after a fixed number of steps.
+
+The ring of the Lanczos vectors is taken up in chunks of 32 steps (or of the
+step cap plus one when that is smaller), so the step counts lie at the edges of
+a chunk; the widths leave ragged 16-byte chunks of columns and ragged column
+blocks; the node counts reach each instance of the pass over the ring (1, 2,
+4, 8 and two passes). solve_tol = 0: every system runs to the cap.
+
+Tolerance (backward errors): a step rounds each value a few times (2^2), which
+is an error of the matrix of at most 2^2 eps ||A|| per step; k <= 70 steps make
+2^2 k < 2^9 of it. It changes x_j = (z_j - A)^-1 q by at most
+2^9 eps ||A|| / Im(z_j) times ||x_j|| <= ||q|| / Im(z_j), so the error of a
+column of unit norm is at most
+2^9 eps ||A|| sum_j |w_j| / Im(z_j)^2. On a grid no Ritz value converges within
+these steps, so the recurrence itself amplifies nothing.
+"""
+import numpy as np
+import pytest
+
+from gpu_util import colmajor_dev, from_colmajor
+from oracle import feast as OF
+from oracle import quadrature as OQ
+from workloads import graphs as G
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("values_free", [0, 1])
+@pytest.mark.parametrize("steps", [1, 31, 32, 33, 70])
+@pytest.mark.parametrize("m0,nc", [(1, 1), (5, 2), (46, 3), (80, 4), (17, 8), (97, 12)])
+def test_fixed_steps_match_oracle(lib, m0, nc, steps, values_free):
+    import torch
+    lap = G.grid2d(37, 41, shift=0.3)
+    A, n, (lo, hi) = lap.scipy(), lap.n, (0.31, 0.6)
+    q0 = OF.random_start(n, m0, 1)
+    z, w = OQ.nodes(lo, hi, nc, 1.0)
+    exp, _ = OF.filter_apply(A, q0, z, w, 0.0, steps, "direct")
+    bound = 2.0 ** 9 * OF.one_norm(A) * np.sum(np.abs(w) / z.imag ** 2)
+    h = lib.rafeast_create(lap.row_ptr, lap.col_idx, lap.values, lap.shift)
+    try:
+        lib.rafeast_set_option(h, lib.RAFEAST_OPT_VALUES_FREE, values_free)
+        for prec, tiled, eps in ((lib.RAFEAST_FP64, 1, 2.0 ** -52), (lib.RAFEAST_MIXED, 1, 2.0 ** -23),
+                                 (lib.RAFEAST_MIXED, 2, 2.0 ** -23)):
+            lib.rafeast_set_option(h, lib.RAFEAST_OPT_TILED, tiled)
+            prm = lib.make_params(lo, hi, m0, nc, 1.0, 0.0, 1e-10, 1, steps, prec,
+                                  lib.RAFEAST_FORM_DIRECT)
+            Q = colmajor_dev(q0)
+            Qt = torch.zeros_like(Q)
+            info = lib.rafeast_filter(h, prm, Q, None, Qt)
+            assert info.cocg_min_last == info.cocg_max_last == steps
+            err = np.linalg.norm(from_colmajor(Qt) - exp, axis=0)
+            assert np.max(err) <= bound * eps, (prec, tiled, float(np.max(err)))
+    finally:
+        lib.rafeast_destroy(h)
+
+
+def test_zero_column_and_nan_input(lib):
+    """A zero column stops at step 0 with a zero result; a NaN column is
+    reported as a breakdown, as by the COCG kernels."""
+    import torch
+    lap = G.grid2d(20, 23, shift=0.3)
+    q0 = OF.random_start(lap.n, 6, 2)
+    q0[:, 2] = 0.0
+    h = lib.rafeast_create(lap.row_ptr, lap.col_idx, lap.values, lap.shift)
+    try:
+        for prec in (lib.RAFEAST_FP64, lib.RAFEAST_MIXED):
+            prm = lib.make_params(0.31, 0.6, 6, 4, 1.0, 1e-3, 1e-10, 1, 200, prec, lib.RAFEAST_FORM_DIRECT)
+            Q = colmajor_dev(q0)
+            Qt = torch.full_like(Q, 7.0)
+            lib.rafeast_filter(h, prm, Q, None, Qt)
+            got = from_colmajor(Qt)
+            assert np.all(got[:, 2] == 0.0) and np.all(np.isfinite(got))
+            Q[4, 5] = float("nan")
+            with pytest.raises(lib.RafeastError) as ei:
+                lib.rafeast_filter(h, prm, Q, None, Qt)
+            assert ei.value.code == lib.RAFEAST_ERR_COCG_BREAKDOWN
+    finally:
+        lib.rafeast_destroy(h)
