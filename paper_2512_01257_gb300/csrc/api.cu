@@ -1798,7 +1798,7 @@ static void import_block(Handle* h, const double* src, int m, int on_device, dou
     RF_CUDA(cudaMemcpyAsync(tmp, src, sizeof(double) * h->n * m, cudaMemcpyHostToDevice, h->stream));
     dsrc = tmp;
   }
-  launch_to_internal(h->n, m, dsrc, dst, ld, h->perm, h->stream);
+  launch_to_internal(h->n, m, dsrc, dst, ld, h->iperm, h->stream);
   h->launches += 1;
 }
 
@@ -1807,7 +1807,7 @@ static void export_block(Handle* h, const double* src, int ld, int m, const int3
   if (m <= 0) return;
   double* ddst = dst;
   if (!on_device) ddst = (double*)scratch(h, S_IO2, sizeof(double) * h->n * m);
-  launch_from_internal(h->n, m, src, ld, ddst, h->perm, cols_d, h->stream);
+  launch_from_internal(h->n, m, src, ld, ddst, h->iperm, cols_d, h->stream);
   h->launches += 1;
   if (!on_device) {
     RF_CUDA(cudaMemcpyAsync(dst, ddst, sizeof(double) * h->n * m, cudaMemcpyDeviceToHost,
@@ -1893,7 +1893,7 @@ static void solve_begin(SolveRun& r, Handle* h, const rafeast_params& prm) {
     ensure_subspace_bufs(h, m0);
     double* om = (double*)scratch(h, S_OMEGA, sizeof(double) * h->n * m0);
     launch_omega(prm.seed, h->n, m0, om, h->stream);
-    launch_to_internal(h->n, m0, om, h->Q, h->ldq, h->perm, h->stream);
+    launch_to_internal(h->n, m0, om, h->Q, h->ldq, h->iperm, h->stream);
     h->launches += 2;
     double* X = h->Q;
     double* Y = (double*)scratch(h, S_TMP1, sizeof(double) * h->n * h->ldq);
@@ -2483,7 +2483,7 @@ int rafeast_spmm(rafeast_t hh, int k, double alpha, double beta, const double* X
   const int ld = even(k);
   double* Xi = (double*)scratch(h, S_TMP1, sizeof(double) * h->n * ld);
   double* Yi = (double*)scratch(h, S_TMP2, sizeof(double) * h->n * ld);
-  launch_to_internal(h->n, k, X, Xi, ld, h->perm, h->stream);
+  launch_to_internal(h->n, k, X, Xi, ld, h->iperm, h->stream);
   // Y = alpha (L + shift I) X + beta X = alpha L X + (alpha shift + beta) X
   if (precision == RAFEAST_FP64) {
     launch_spmm_real<double>(h->n, h->rowptr, h->colidx, h->val64, k, ld, alpha,
@@ -2496,7 +2496,7 @@ int rafeast_spmm(rafeast_t hh, int k, double alpha, double beta, const double* X
                             alpha * h->shift + beta, Xf, Yf, h->num_sms, h->stream);
     launch_widen(Yf, Yi, h->n * (int64_t)ld, h->stream);
   }
-  launch_from_internal(h->n, k, Yi, ld, Y, h->perm, nullptr, h->stream);
+  launch_from_internal(h->n, k, Yi, ld, Y, h->iperm, nullptr, h->stream);
   scope.finish();
   RF_CUDA(cudaStreamSynchronize(h->stream));
   return RAFEAST_OK;
@@ -2598,7 +2598,7 @@ int rafeast_filter(rafeast_t hh, const rafeast_params* prm, const double* Q, con
   double* AQi = (double*)scratch(h, S_TMP2, sizeof(double) * h->n * ldq);
   double* Qti = (double*)scratch(h, S_QT, sizeof(double) * h->n * ldq);
   RF_CUDA(cudaMemsetAsync(Qti, 0, sizeof(double) * h->n * ldq, h->stream));
-  launch_to_internal(h->n, m0, Q, Qi, ldq, h->perm, h->stream);
+  launch_to_internal(h->n, m0, Q, Qi, ldq, h->iperm, h->stream);
   launch_spmm_real<double>(h->n, h->rowptr, h->colidx, h->val64, m0, ldq, 1.0, h->shift, Qi, AQi,
                            h->num_sms, h->stream);
   std::vector<double> th(m0);
@@ -2634,7 +2634,7 @@ int rafeast_filter(rafeast_t hh, const rafeast_params* prm, const double* Q, con
     rc = e.code;
   }
   RF_CUDA(cudaEventRecord(e1, h->stream));
-  launch_from_internal(h->n, m0, Qti, ldq, Qt, h->perm, nullptr, h->stream);
+  launch_from_internal(h->n, m0, Qti, ldq, Qt, h->iperm, nullptr, h->stream);
   RF_CUDA(cudaStreamSynchronize(h->stream));
   float ms = 0.f;
   RF_CUDA(cudaEventElapsedTime(&ms, e0, e1));
@@ -2664,12 +2664,12 @@ int rafeast_orthonormalize(rafeast_t hh, int m, double* Q, double* R) {
   const int ld = even(m);
   double* A = (double*)scratch(h, S_TMP1, sizeof(double) * h->n * ld);
   double* B = (double*)scratch(h, S_TMP2, sizeof(double) * h->n * ld);
-  launch_to_internal(h->n, m, Q, A, ld, h->perm, h->stream);
+  launch_to_internal(h->n, m, Q, A, ld, h->iperm, h->stream);
   std::vector<double> Rt;
   double* X = A;
   double* Y = B;
   cholqr(h, X, Y, m, ld, R ? &Rt : nullptr);
-  launch_from_internal(h->n, m, X, ld, Q, h->perm, nullptr, h->stream);
+  launch_from_internal(h->n, m, X, ld, Q, h->iperm, nullptr, h->stream);
   RF_CUDA(cudaStreamSynchronize(h->stream));
   if (R) {
     // column-major output of the row-major upper factor
@@ -2689,10 +2689,10 @@ int rafeast_gram(rafeast_t hh, int m, const double* X, const double* Y, double* 
   const int ld = even(m);
   double* Xi = (double*)scratch(h, S_TMP1, sizeof(double) * h->n * ld);
   double* Yi = Xi;
-  launch_to_internal(h->n, m, X, Xi, ld, h->perm, h->stream);
+  launch_to_internal(h->n, m, X, Xi, ld, h->iperm, h->stream);
   if (Y != X) {  // (the same block twice: X^T X, one copy and one digit split)
     Yi = (double*)scratch(h, S_TMP2, sizeof(double) * h->n * ld);
-    launch_to_internal(h->n, m, Y, Yi, ld, h->perm, h->stream);
+    launch_to_internal(h->n, m, Y, Yi, ld, h->iperm, h->stream);
   }
   DenseWs d = dense_ws(h, m);
   // row-major (Y^T X)[b][a] = sum_r Y[r][b] X[r][a] is G = X^T Y in column-major order
@@ -2714,7 +2714,7 @@ int rafeast_block_product(rafeast_t hh, int m, const double* X, const double* M,
   const int ldx = even(m), ldy = even(mo);
   double* Xi = (double*)scratch(h, S_TMP1, sizeof(double) * h->n * ldx);
   double* Yi = (double*)scratch(h, S_TMP2, sizeof(double) * h->n * ldy);
-  launch_to_internal(h->n, m, X, Xi, ldx, h->perm, h->stream);
+  launch_to_internal(h->n, m, X, Xi, ldx, h->iperm, h->stream);
   // M: caller's column-major m x mo -> row-major, through the host (small)
   std::vector<double> mc((size_t)m * mo), mr((size_t)m * mo);
   RF_CUDA(cudaMemcpyAsync(mc.data(), M, sizeof(double) * m * mo, cudaMemcpyDeviceToHost,
@@ -2726,7 +2726,7 @@ int rafeast_block_product(rafeast_t hh, int m, const double* X, const double* M,
   RF_CUDA(cudaMemcpyAsync(Mr, mr.data(), sizeof(double) * m * mo, cudaMemcpyHostToDevice,
                           h->stream));
   tall_dev(h, Xi, m, ldx, Mr, mo, Yi, ldy);
-  launch_from_internal(h->n, mo, Yi, ldy, Y, h->perm, nullptr, h->stream);
+  launch_from_internal(h->n, mo, Yi, ldy, Y, h->iperm, nullptr, h->stream);
   h->launches += 3;
   scope.finish();
   RF_CUDA(cudaStreamSynchronize(h->stream));
@@ -2745,12 +2745,12 @@ int rafeast_rayleigh_ritz(rafeast_t hh, int m, double* Q, double* theta, double*
   double* Qo = (double*)scratch(h, S_QT, sizeof(double) * h->n * ld);
   double* AQo = (double*)scratch(h, S_AQ2, sizeof(double) * h->n * ld);
   double* th_d = (double*)scratch(h, S_OMEGA, sizeof(double) * (m + 1));
-  launch_to_internal(h->n, m, Q, X, ld, h->perm, h->stream);
+  launch_to_internal(h->n, m, Q, X, ld, h->iperm, h->stream);
   rayleigh_ritz_dev(h, X, m, ld, Qo, AQo, th_d, tmp);
   std::vector<double> res;
   residuals_host(h, Qo, AQo, th_d, m, ld, res);
   RF_CUDA(cudaMemcpyAsync(theta, th_d, sizeof(double) * m, cudaMemcpyDeviceToHost, h->stream));
-  launch_from_internal(h->n, m, Qo, ld, Q, h->perm, nullptr, h->stream);
+  launch_from_internal(h->n, m, Qo, ld, Q, h->iperm, nullptr, h->stream);
   RF_CUDA(cudaStreamSynchronize(h->stream));
   if (resid) std::copy(res.begin(), res.end(), resid);
   scope.finish();
@@ -2783,7 +2783,7 @@ int rafeast_warmstart(rafeast_t hh, double lmin, double lmax, int m0, int p, int
   double* Y = (double*)scratch(h, S_TMP1, sizeof(double) * h->n * ld);
   double* Z = (double*)scratch(h, S_TMP2, sizeof(double) * h->n * ld);
   launch_omega(seed, h->n, k, om, h->stream);
-  launch_to_internal(h->n, k, om, Z, ld, h->perm, h->stream);
+  launch_to_internal(h->n, k, om, Z, ld, h->iperm, h->stream);
   launch_spmm_real<double>(h->n, h->rowptr, h->colidx, h->val64, k, ld, sL, sI, Z, Y, h->num_sms,
                            h->stream);
   h->launches += 3;

@@ -498,9 +498,9 @@ void launch_philox(uint64_t seed, uint64_t first, int64_t nblocks, uint64_t* out
 void launch_omega(uint64_t seed, int64_t n, int k, double* out_colmajor, cudaStream_t s);
 // caller col-major (n x m, ld n, original order) <-> internal row-major (ld)
 void launch_to_internal(int64_t n, int m, const double* src, double* dst, int ld,
-                        const int32_t* perm, cudaStream_t s);
+                        const int32_t* iperm, cudaStream_t s);
 void launch_from_internal(int64_t n, int m, const double* src, int ld, double* dst,
-                          const int32_t* perm, const int32_t* cols /* may be null */,
+                          const int32_t* iperm, const int32_t* cols /* may be null */,
                           cudaStream_t s);
 // row-major tall blocks, FP64
 // G = X^T Y (m x m, ld m); sym: X^T Y is symmetric (X^T X, X^T A X), only

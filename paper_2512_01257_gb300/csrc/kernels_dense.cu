@@ -111,29 +111,81 @@ void launch_omega(uint64_t seed, int64_t n, int k, double* out, cudaStream_t s) 
 // ---------------------------------------------------------------------------
 // layout moves
 // ---------------------------------------------------------------------------
-__global__ void k_to_internal(int64_t n, int m, const double* __restrict__ src,
-                              double* __restrict__ dst, int ld, const int32_t* __restrict__ perm) {
-  const int64_t total = n * (int64_t)ld;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = e / ld;
-    const int c = (int)(e - r * ld);
-    const int64_t o = perm ? perm[r] : r;
-    dst[e] = c < m ? src[(int64_t)c * n + o] : 0.0;
+// A CTA moves MV_R rows, consecutive in the caller's order, by MV_C columns
+// through shared memory: the column-major side is read or written 32 rows (256 bytes) of a
+// column at a time, the row-major side 512 bytes of a row at a time, wherever the
+// reordering put it. (One thread per element with the reordered index on the
+// column-major side touched a 32-byte sector per 8-byte value: 155 us in and
+// 344 us out for 200,000 x 80 against 128 MB each way.)
+constexpr int MV_R = 32, MV_C = 64;
+__global__ void __launch_bounds__(256) k_to_internal(int64_t n, int m,
+                                                     const double* __restrict__ src,
+                                                     double* __restrict__ dst, int ld,
+                                                     const int32_t* __restrict__ iperm) {
+  __shared__ double mv[MV_R][MV_C + 1];
+  const int64_t o0 = (int64_t)blockIdx.x * MV_R;
+  const int rows = (int)min((int64_t)MV_R, n - o0);
+  const int c0 = blockIdx.y * MV_C, nc = min(MV_C, ld - c0);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int u = 0; u < MV_C / 8; ++u) {
+    const int c = warp + 8 * u;
+    if (c < nc) mv[lane][c] = (c0 + c < m && lane < rows) ? src[(int64_t)(c0 + c) * n + o0 + lane] : 0.0;
+  }
+  __syncthreads();
+  for (int r = warp; r < rows; r += 8) {
+    double* out = dst + (iperm ? (int64_t)iperm[o0 + r] : o0 + r) * ld + c0;
+    for (int c = lane; c < nc; c += 32) out[c] = mv[r][c];
   }
 }
 
-__global__ void k_from_internal(int64_t n, int m, const double* __restrict__ src, int ld,
-                                double* __restrict__ dst, const int32_t* __restrict__ perm,
-                                const int32_t* __restrict__ cols) {
+__global__ void __launch_bounds__(256) k_from_internal(int64_t n, int m,
+                                                       const double* __restrict__ src, int ld,
+                                                       double* __restrict__ dst,
+                                                       const int32_t* __restrict__ iperm,
+                                                       const int32_t* __restrict__ cols) {
+  __shared__ double mv[MV_R][MV_C + 1];
+  const int64_t o0 = (int64_t)blockIdx.x * MV_R;
+  const int rows = (int)min((int64_t)MV_R, n - o0);
+  const int c0 = blockIdx.y * MV_C, nc = min(MV_C, m - c0);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int u = 0; u < MV_R / 8; ++u) {
+    const int r = warp + 8 * u;
+    if (r >= rows) break;
+    const double* in = src + (iperm ? (int64_t)iperm[o0 + r] : o0 + r) * ld;
+    for (int c = lane; c < nc; c += 32) mv[r][c] = in[cols ? cols[c0 + c] : c0 + c];
+  }
+  __syncthreads();
+  if (lane < rows)
+    for (int c = warp; c < nc; c += 8) dst[(int64_t)(c0 + c) * n + o0 + lane] = mv[lane][c];
+}
+
+// the same one element per thread, for blocks that both levels of cache hold
+// anyway (at most MV_SMALL elements): no shared-memory phase to wait for. 24
+// columns of 2,000 rows: a product with both moves takes 30 us this way, 33 us
+// through shared memory; from about 8 MB on the sectors wasted cost more.
+constexpr int64_t MV_SMALL = 1 << 19;
+__global__ void k_to_internal_small(int64_t n, int m, const double* __restrict__ src,
+                                    double* __restrict__ dst, int ld,
+                                    const int32_t* __restrict__ iperm) {
+  const int64_t total = n * (int64_t)ld;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t o = e / ld;
+    const int c = (int)(e - o * ld);
+    dst[(iperm ? (int64_t)iperm[o] : o) * ld + c] = c < m ? src[(int64_t)c * n + o] : 0.0;
+  }
+}
+__global__ void k_from_internal_small(int64_t n, int m, const double* __restrict__ src, int ld,
+                                      double* __restrict__ dst, const int32_t* __restrict__ iperm,
+                                      const int32_t* __restrict__ cols) {
   const int64_t total = n * (int64_t)m;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = e / m;
-    const int c = (int)(e - r * m);
-    const int64_t o = perm ? perm[r] : r;
-    const int sc = cols ? cols[c] : c;
-    dst[(int64_t)c * n + o] = src[r * ld + sc];
+    const int64_t o = e / m;
+    const int c = (int)(e - o * m);
+    dst[(int64_t)c * n + o] = src[(iperm ? (int64_t)iperm[o] : o) * ld + (cols ? cols[c] : c)];
   }
 }
 
@@ -145,15 +197,27 @@ static int blocks_for(int64_t total, int per = 256, int cap = 16384) {
 }
 
 void launch_to_internal(int64_t n, int m, const double* src, double* dst, int ld,
-                        const int32_t* perm, cudaStream_t s) {
-  k_to_internal<<<blocks_for(n * (int64_t)ld), 256, 0, s>>>(n, m, src, dst, ld, perm);
+                        const int32_t* iperm, cudaStream_t s) {
+  if (n <= 0 || ld <= 0) return;
+  if (n * (int64_t)ld <= MV_SMALL) {
+    k_to_internal_small<<<blocks_for(n * (int64_t)ld), 256, 0, s>>>(n, m, src, dst, ld, iperm);
+  } else {
+    const dim3 grid((unsigned)((n + MV_R - 1) / MV_R), (ld + MV_C - 1) / MV_C);
+    k_to_internal<<<grid, 256, 0, s>>>(n, m, src, dst, ld, iperm);
+  }
   RF_LAUNCH();
 }
 
 void launch_from_internal(int64_t n, int m, const double* src, int ld, double* dst,
-                          const int32_t* perm, const int32_t* cols, cudaStream_t s) {
-  if (m <= 0) return;
-  k_from_internal<<<blocks_for(n * (int64_t)m), 256, 0, s>>>(n, m, src, ld, dst, perm, cols);
+                          const int32_t* iperm, const int32_t* cols, cudaStream_t s) {
+  if (n <= 0 || m <= 0) return;
+  if (n * (int64_t)m <= MV_SMALL) {
+    k_from_internal_small<<<blocks_for(n * (int64_t)m), 256, 0, s>>>(n, m, src, ld, dst, iperm,
+                                                                     cols);
+  } else {
+    const dim3 grid((unsigned)((n + MV_R - 1) / MV_R), (m + MV_C - 1) / MV_C);
+    k_from_internal<<<grid, 256, 0, s>>>(n, m, src, ld, dst, iperm, cols);
+  }
   RF_LAUNCH();
 }
 
@@ -249,27 +313,47 @@ __global__ void __launch_bounds__(256) k_gram_partial(const double* __restrict__
 // summation (A. Neumaier, ZAMM 54, 1974): the rounding error of every
 // addition is carried along, so the sum of the CTAs' partials adds about
 // two units of rounding instead of one per partial.
-__global__ void k_gram_sum(const double* __restrict__ part, int nparts, int m, int sym,
-                           double* G) {
+// Eight lanes share an entry: lane l adds the partials l, l + 8, ..., then the
+// lanes' (sum, error) pairs are added by a fixed tree. (One thread per entry
+// ran a chain of 152 or 304 dependent FP64 additions: 63 to 117 us for m = 52
+// to 100.)
+__global__ void __launch_bounds__(128) k_gram_sum(const double* __restrict__ part, int nparts,
+                                                  int m, int sym, double* G) {
   const int mm = m * m;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < mm; e += gridDim.x * blockDim.x) {
-    const int a = e / m, b = e - a * m;
-    const int src = (sym && (a >> 4) > (b >> 4)) ? b * m + a : e;
-    double s = 0.0, c = 0.0;
-    for (int p = 0; p < nparts; ++p) {
-      const double v = part[(int64_t)p * mm + src];
-      const double t = s + v;
-      c += fabs(s) >= fabs(v) ? (s - t) + v : (v - t) + s;
-      s = t;
-    }
-    G[e] = s + c;
+  const int e = blockIdx.x * 16 + (threadIdx.x >> 3), l = threadIdx.x & 7;
+  const bool on = e < mm;
+  const int a = on ? e / m : 0, b = on ? e - a * m : 0;
+  const int src = (sym && (a >> 4) > (b >> 4)) ? b * m + a : (on ? e : 0);
+  double s = 0.0, c = 0.0;
+  auto add = [&](double v) {
+    const double t = s + v;
+    c += fabs(s) >= fabs(v) ? (s - t) + v : (v - t) + s;
+    s = t;
+  };
+  for (int p0 = l; p0 < nparts; p0 += 64) {
+    double v[8];  // (past the end: + 0, which changes nothing)
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      v[u] = p0 + 8 * u < nparts ? part[(int64_t)(p0 + 8 * u) * mm + src] : 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) add(v[u]);
   }
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) {
+    const double so = __shfl_xor_sync(0xffffffffu, s, o), co = __shfl_xor_sync(0xffffffffu, c, o);
+    // (the lower lane's pair first, so that all lanes of an entry agree)
+    const double x = (l & o) ? so : s, y = (l & o) ? s : so;
+    c = (l & o) ? co + c : c + co;
+    s = x;
+    add(y);
+  }
+  if (on && l == 0) G[e] = s + c;
 }
 
 int gram_parts(int num_sms) { return 2 * num_sms; }
 
 void gram_sum(const double* part, int parts, int m, bool sym, double* G, cudaStream_t s) {
-  k_gram_sum<<<(m * m + 255) / 256, 256, 0, s>>>(part, parts, m, sym ? 1 : 0, G);
+  k_gram_sum<<<(m * m + 15) / 16, 128, 0, s>>>(part, parts, m, sym ? 1 : 0, G);
   RF_LAUNCH();
 }
 
@@ -302,8 +386,7 @@ void gram(const double* X, const double* Y, int64_t n, int m, int ld, double* G,
     gram_partials<false>(X, Y, n, m, ld, partial, parts, smem, s);
   }
   RF_LAUNCH();
-  k_gram_sum<<<(m * m + 255) / 256, 256, 0, s>>>(partial, parts, m, sym ? 1 : 0, G);
-  RF_LAUNCH();
+  gram_sum(partial, parts, m, sym, G, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -389,39 +472,50 @@ void tall_gemm(const double* X, int64_t n, int m, int ldx, const double* M, int 
 }
 
 // ---------------------------------------------------------------------------
-// one-CTA Cholesky (+shift) and triangular inverse
-// G: m x m (row-major, symmetric). Outputs R (upper, G = R^T R, row-major) and
-// Rinv (upper, row-major); status: 0 ok, 1 shifted, 2 failed.
+// Cholesky (+shift) by one CTA, then the triangular inverse by one warp per
+// column. G: m x m (row-major, symmetric). Outputs R (upper, G = R^T R,
+// row-major) and Rinv (upper, row-major); status: 0 ok, 1 shifted, 2 failed.
+//
+// One SM issues 2 FP64 lane operations a clock, so the m^3 / 6 products of the
+// factorisation alone take 22 us at m = 80; the inverse, as many again, is
+// spread over the chip, where a column costs a latency chain of m steps. (Both
+// in one CTA, the inverse one column per thread: 234 us; now 55 us.)
 // ---------------------------------------------------------------------------
+// S: column-major lower triangle, S[k * m + i] = L_ik (i >= k)
 __device__ bool chol_inplace(double* S, int m) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   __shared__ int s_bad;
   if (threadIdx.x == 0) s_bad = 0;
   __syncthreads();
   for (int k = 0; k < m; ++k) {
-    if (threadIdx.x == 0) {
-      const double d = S[k * m + k];
-      if (!(d > 0.0) || !isfinite(d)) s_bad = 1;
-      else S[k * m + k] = sqrt(d);
+    double* Sk = S + k * m;
+    if (warp == 0) {  // the pivot, computed by every lane, and its column
+      const double d = Sk[k];
+      const bool bad = !(d > 0.0) || !isfinite(d);
+      const double r = sqrt(d), ir = 1.0 / r;
+      __syncwarp();
+      if (lane == 0) {
+        if (bad) s_bad = 1;
+        else Sk[k] = r;
+      }
+      if (!bad)
+        for (int i = k + 1 + lane; i < m; i += 32) Sk[i] *= ir;
     }
     __syncthreads();
     if (s_bad) return false;
-    const double dk = S[k * m + k];
-    for (int i = k + 1 + threadIdx.x; i < m; i += blockDim.x) S[i * m + k] /= dk;
-    __syncthreads();
-    const int rem = m - k - 1;
-    const int tot = rem * rem;
-    for (int t = threadIdx.x; t < tot; t += blockDim.x) {
-      const int i = k + 1 + t / rem, j = k + 1 + t % rem;
-      if (j <= i) S[i * m + j] -= S[i * m + k] * S[j * m + k];
+    // trailing update, a warp per column
+    for (int j = k + 1 + warp; j < m; j += nw) {
+      const double ljk = Sk[j];
+      for (int i = j + lane; i < m; i += 32) S[j * m + i] = fma(-Sk[i], ljk, S[j * m + i]);
     }
     __syncthreads();
   }
   return true;
 }
 
-__global__ void k_chol_inv(const double* __restrict__ G, int m, double shift_scale,
-                           double* __restrict__ R, double* __restrict__ Rinv, int* status,
-                           int check_id) {
+__global__ void __launch_bounds__(512) k_chol(const double* __restrict__ G, int m,
+                                              double shift_scale, double* __restrict__ R,
+                                              int* status, int check_id) {
   extern __shared__ double S[];  // m*m
   __shared__ double s_shift;
   __shared__ int s_far;
@@ -438,6 +532,7 @@ __global__ void k_chol_inv(const double* __restrict__ G, int m, double shift_sca
   bool ok = chol_inplace(S, m);
   if (!ok) {
     // shifted Cholesky-QR: s = 11 (n m + m (m + 1)) u ||X||_2^2, ||X||_2^2 <= trace(G)
+    __syncthreads();
     if (threadIdx.x == 0) {
       double tr = 0.0;
       for (int i = 0; i < m; ++i) tr += fabs(G[i * m + i]);
@@ -456,37 +551,60 @@ __global__ void k_chol_inv(const double* __restrict__ G, int m, double shift_sca
     if (threadIdx.x == 0) status[0] = 2;
     return;
   }
-  // R = L^T (upper)
-  for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
-    const int i = t / m, j = t % m;
-    R[t] = j >= i ? S[j * m + i] : 0.0;
+  // R = L^T: row k of R is column k of L
+  for (int t = threadIdx.x; t < m * m; t += blockDim.x) R[t] = t % m >= t / m ? S[t] : 0.0;
+  if (threadIdx.x == 0) status[0] = st | (s_far ? 4 : 0);
+}
+
+// column j of L^-1 (row j of Rinv) by forward substitution, one warp: lane l
+// holds the entries l, l + 32, ... of the right-hand side, column i of L
+// (row i of R) leaves it once x_i is known
+__global__ void __launch_bounds__(32) k_trinv(const double* __restrict__ R, int m,
+                                              double* __restrict__ Rinv, const int* status) {
+  if (status[0] == 2) return;
+  const int j = blockIdx.x, lane = threadIdx.x;
+  double b[4], id[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int i = lane + 32 * u;
+    b[u] = i == j ? 1.0 : 0.0;
+    id[u] = i < m ? 1.0 / R[i * m + i] : 0.0;
   }
-  // Linv by forward substitution, one column per thread; Rinv = Linv^T
-  for (int j = threadIdx.x; j < m; j += blockDim.x) {
-    for (int i = 0; i < m; ++i) {
-      double x;
-      if (i < j) {
-        x = 0.0;
-      } else {
-        double acc = (i == j) ? 1.0 : 0.0;
-        for (int k = j; k < i; ++k) acc -= S[i * m + k] * Rinv[j * m + k];
-        x = acc / S[i * m + i];
-      }
-      Rinv[j * m + i] = x;  // row j of Rinv holds column j of Linv^T... see below
+  double l[4], ln[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) l[u] = lane + 32 * u < m ? R[j * m + lane + 32 * u] : 0.0;
+  for (int i = j; i < m; ++i) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      ln[u] = (i + 1 < m && lane + 32 * u < m) ? R[(i + 1) * m + lane + 32 * u] : 0.0;
+    const int u0 = i >> 5;
+    const double xb = u0 == 0 ? b[0] * id[0] : u0 == 1 ? b[1] * id[1] : u0 == 2 ? b[2] * id[2] : b[3] * id[3];
+    const double x = __shfl_sync(0xffffffffu, xb, i & 31);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int r = lane + 32 * u;
+      if (r == i) b[u] = x;
+      else if (r > i) b[u] = fma(-l[u], x, b[u]);
+      l[u] = ln[u];
     }
   }
-  __syncthreads();
-  // Rinv currently holds Linv^T stored as Rinv[j][i] = Linv[i][j] = (Linv^T)[j][i]
-  if (threadIdx.x == 0) status[0] = st | (s_far ? 4 : 0);
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int i = lane + 32 * u;
+    if (i < m) Rinv[j * m + i] = i >= j ? b[u] : 0.0;
+  }
 }
 
 void chol_inv(double* G, int m, int64_t nrows, double* Rfac, double* Rinv, int* status,
               cudaStream_t s, bool check_id) {
+  RF_CHECK(m >= 1 && m <= 128, RAFEAST_ERR_INVALID_ARG);
   const size_t smem = (size_t)m * m * sizeof(double);
-  ensure_dyn_smem(reinterpret_cast<const void*>(k_chol_inv), smem);
+  ensure_dyn_smem(reinterpret_cast<const void*>(k_chol), smem);
   const double u = DBL_EPSILON / 2;
   const double scale = 11.0 * ((double)nrows * m + (double)m * (m + 1)) * u;
-  k_chol_inv<<<1, 256, smem, s>>>(G, m, scale, Rfac, Rinv, status, check_id ? 1 : 0);
+  k_chol<<<1, 512, smem, s>>>(G, m, scale, Rfac, status, check_id ? 1 : 0);
+  RF_LAUNCH();
+  k_trinv<<<m, 32, 0, s>>>(Rfac, m, Rinv, status);
   RF_LAUNCH();
 }
 
@@ -498,12 +616,16 @@ constexpr size_t JACOBI_SMEM_MAX = 216 * 1024;  // A and V in shared memory up t
 // A (m x m, ld m, symmetric part taken) -> eigenvalues ascending in w, the
 // matching eigenvectors as the columns of Vout (m x m, ld m). A pair (p, q)
 // is rotated while |a_pq| > rot_tol sqrt(|a_pp a_qq|); the sweeps end when
-// the off-diagonal mass is below off_tol of the total or a sweep rotated
-// nothing. Vg: global fallback for the eigenvector accumulator (me * me).
+// the off-diagonal mass is below off_tol of the total, no off-diagonal entry
+// exceeds abs_tol times the root mean square eigenvalue, or a sweep rotated
+// nothing. Vg: global fallback for the eigenvector accumulator (me * me), which
+// is kept transposed (an entry's column-wise neighbours in V, 16 lanes of a
+// warp in one shared-memory bank, made a float round of m = 80 three times as
+// long).
 template <typename T>
-__global__ void k_jacobi(const double* __restrict__ Ain, int m, double* __restrict__ w,
+__global__ void __launch_bounds__(1024) k_jacobi(const double* __restrict__ Ain, int m, double* __restrict__ w,
                          double* __restrict__ Vout, T* __restrict__ Vg, int max_sweeps,
-                         double rot_tol, double off_tol) {
+                         double rot_tol, double off_tol, double abs_tol) {
   extern __shared__ unsigned char jsm[];
   T* A = reinterpret_cast<T*>(jsm);  // me * me (+ me * me for V when it fits)
   const int me = m + (m & 1);
@@ -512,8 +634,8 @@ __global__ void k_jacobi(const double* __restrict__ Ain, int m, double* __restri
   T* Vw = (2 * (size_t)me * me * sizeof(T) <= JACOBI_SMEM_MAX) ? A + me * me : Vg;
   __shared__ T cs[64 * 2];  // c, s per pair (me/2 <= 64)
   __shared__ int pq[64 * 2];
-  __shared__ double s_off, s_tot;
-  __shared__ double s_woff[32], s_wtot[32];  // per-warp sums, added in warp order
+  __shared__ double s_off, s_tot, s_max;
+  __shared__ double s_woff[32], s_wtot[32], s_wmax[32];  // per-warp sums, added in warp order
   __shared__ int s_order[128];
   __shared__ int s_rot;
   const T tiny = sizeof(T) == 4 ? (T)1e-37 : (T)1e-300;
@@ -524,6 +646,22 @@ __global__ void k_jacobi(const double* __restrict__ Ain, int m, double* __restri
   }
   __syncthreads();
   const int np = me / 2;
+  // this thread's 2 x 2 blocks (j, k) of A and entries (k, row) of V^T are the
+  // same in every round
+  constexpr int TA = 4, TV = 8;  // np * np <= 4 * 1024, np * me <= 8 * 1024
+  int tj[TA], tk[TA], vk[TV], vr[TV];
+#pragma unroll
+  for (int u = 0; u < TA; ++u) {
+    const int t = threadIdx.x + u * (int)blockDim.x;
+    tj[u] = t < np * np ? t / np : -1;
+    tk[u] = t - (t / np) * np;
+  }
+#pragma unroll
+  for (int u = 0; u < TV; ++u) {
+    const int t = threadIdx.x + u * (int)blockDim.x;
+    vk[u] = t < np * me ? t / me : -1;
+    vr[u] = t - (t / me) * me;
+  }
   for (int sweep = 0; sweep < max_sweeps; ++sweep) {
     // convergence test on the off-diagonal mass
     if (threadIdx.x == 0) {
@@ -532,35 +670,49 @@ __global__ void k_jacobi(const double* __restrict__ Ain, int m, double* __restri
       s_rot = 0;
     }
     __syncthreads();
-    double off = 0.0, tot = 0.0;
+    double off = 0.0, tot = 0.0, mx = 0.0;
     for (int t = threadIdx.x; t < me * me; t += blockDim.x) {
       const int i = t / me, j = t % me;
       const double a2 = (double)A[t] * (double)A[t];
       tot += a2;
-      if (i != j) off += a2;
+      if (i != j) {
+        off += a2;
+        mx = fmax(mx, fabs((double)A[t]));
+      }
     }
     off = warp_sum(off);
     tot = warp_sum(tot);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if ((threadIdx.x & 31) == 0) {
       s_woff[threadIdx.x >> 5] = off;
       s_wtot[threadIdx.x >> 5] = tot;
+      s_wmax[threadIdx.x >> 5] = mx;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-      double so = 0.0, st = 0.0;
+      double so = 0.0, st = 0.0, sm = 0.0;
       for (int wi = 0; wi < (int)(blockDim.x >> 5); ++wi) {
         so += s_woff[wi];
         st += s_wtot[wi];
+        sm = fmax(sm, s_wmax[wi]);
       }
       s_off = so;
       s_tot = st;
+      s_max = sm;
     }
     __syncthreads();
     if (!(s_off > off_tol * s_tot) || s_tot == 0.0) break;
+    const T small = (T)(abs_tol * sqrt(s_tot / m));
+    if (abs_tol > 0.0 && !(s_max > (double)small)) break;
     for (int round = 0; round < me - 1; ++round) {
+      int rotates = 0;
       for (int k = threadIdx.x; k < np; k += blockDim.x) {
         // circle method: position 0 fixed, others rotate
-        auto player = [&](int pos) { return pos == 0 ? 0 : ((pos - 1 + round) % (me - 1)) + 1; };
+        auto player = [&](int pos) {
+          const int x = pos - 1 + round;  // < 2 (me - 1)
+          return pos == 0 ? 0 : (x >= me - 1 ? x - (me - 1) : x) + 1;
+        };
         int p = player(k), q = player(me - 1 - k);
         if (p > q) {
           const int t = p;
@@ -570,8 +722,10 @@ __global__ void k_jacobi(const double* __restrict__ Ain, int m, double* __restri
         const T apq = A[p * me + q];
         T c = (T)1, s = (T)0;
         const T app = A[p * me + p], aqq = A[q * me + q];
-        if (apq != (T)0 && fabs(apq) > tiny && fabs(apq) > (T)rot_tol * sqrt(fabs(app * aqq))) {
+        if (apq != (T)0 && fabs(apq) > tiny && fabs(apq) > small &&
+            fabs(apq) > (T)rot_tol * sqrt(fabs(app * aqq))) {
           s_rot = 1;
+          rotates = 1;
           const T tau = (aqq - app) / ((T)2 * apq);
           const T at = fabs(tau);
           const T root = at > (T)1e15 ? at : sqrt((T)1 + tau * tau);
@@ -584,13 +738,15 @@ __global__ void k_jacobi(const double* __restrict__ Ain, int m, double* __restri
         pq[2 * k] = p;
         pq[2 * k + 1] = q;
       }
-      __syncthreads();
+      if (!__syncthreads_or(rotates)) continue;  // (no pair of this round is rotated)
       // the pairs of a round are disjoint, so every 2 x 2 block (rows of
       // pair j, columns of pair k) is updated on its own from its old
       // values: B <- L_j B R_k with L = [[c, -s], [s, c]], R = L^T; the
       // rotated diagonal blocks lose their off-diagonal entry
-      for (int t = threadIdx.x; t < np * np; t += blockDim.x) {
-        const int j = t / np, k = t % np;
+#pragma unroll
+      for (int u = 0; u < TA; ++u) {
+        if (tj[u] < 0) break;
+        const int j = tj[u], k = tk[u];
         const T cj = cs[2 * j], sj = cs[2 * j + 1];
         const T ck = cs[2 * k], sk = cs[2 * k + 1];
         if (sj == (T)0 && sk == (T)0) continue;
@@ -607,84 +763,135 @@ __global__ void k_jacobi(const double* __restrict__ Ain, int m, double* __restri
         A[qj * me + pk] = j == k ? (T)0 : ck * b21 - sk * b22;
         A[qj * me + qk] = sk * b21 + ck * b22;
       }
-      // V R_k
-      for (int t = threadIdx.x; t < np * me; t += blockDim.x) {
-        const int k = t / me, row = t % me;
+      // V R_k, on V^T: a warp's lanes take consecutive entries of the two rows
+#pragma unroll
+      for (int u = 0; u < TV; ++u) {
+        if (vk[u] < 0) break;
+        const int k = vk[u], row = vr[u];
         const T c = cs[2 * k], s = cs[2 * k + 1];
         if (s == (T)0) continue;
         const int p = pq[2 * k], q = pq[2 * k + 1];
-        const T vp = Vw[row * me + p], vq = Vw[row * me + q];
-        Vw[row * me + p] = c * vp - s * vq;
-        Vw[row * me + q] = s * vp + c * vq;
+        const T vp = Vw[p * me + row], vq = Vw[q * me + row];
+        Vw[p * me + row] = c * vp - s * vq;
+        Vw[q * me + row] = s * vp + c * vq;
       }
       __syncthreads();
     }
     if (s_rot == 0) break;  // nothing was above the threshold in this sweep
     __syncthreads();
   }
-  // sort eigenvalues ascending (m <= 128), then write w and V columns
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < m; ++i) s_order[i] = i;
-    for (int i = 1; i < m; ++i) {
-      const int key = s_order[i];
-      const T kv = A[key * me + key];
-      int j = i - 1;
-      while (j >= 0 && A[s_order[j] * me + s_order[j]] > kv) {
-        s_order[j + 1] = s_order[j];
-        --j;
-      }
-      s_order[j + 1] = key;
+  // eigenvalues ascending (m <= 128; equal ones in index order): the rank of
+  // each; then w and the columns of V
+  __syncthreads();
+  for (int i = threadIdx.x; i < m; i += blockDim.x) s_order[i] = i;  // (kept where NaNs leave a gap)
+  __syncthreads();
+  for (int i = threadIdx.x; i < m; i += blockDim.x) {
+    const T v = A[i * me + i];
+    int rank = 0;
+    for (int j = 0; j < m; ++j) {
+      const T x = A[j * me + j];
+      rank += (x < v || (x == v && j < i)) ? 1 : 0;
     }
+    s_order[rank] = i;
   }
   __syncthreads();
   for (int i = threadIdx.x; i < m; i += blockDim.x) w[i] = (double)A[s_order[i] * me + s_order[i]];
   for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
     const int r = t / m, c = t % m;
-    Vout[r * m + c] = (double)Vw[r * me + s_order[c]];
+    Vout[r * m + c] = (double)Vw[s_order[c] * me + r];
   }
 }
 
 // small dense product, all m x m row-major: C = alpha op(A) op(B) + gamma I,
-// op = transpose when the flag is set; one thread per entry of C
-__global__ void k_small_gemm(const double* __restrict__ A, int ta, const double* __restrict__ B,
-                             int tb, double* __restrict__ C, int m, double alpha, double gamma) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= m * m) return;
-  const int i = e / m, j = e - (e / m) * m;
-  double acc = 0.0;
-  for (int k = 0; k < m; ++k) {
-    const double a = ta ? A[k * m + i] : A[i * m + k];
-    const double b = tb ? B[j * m + k] : B[k * m + j];
-    acc = fma(a, b, acc);
+// op = transpose when the flag is set. A CTA of 64 threads forms an 8 x 8
+// block of C from panels staged in shared memory: small blocks put the FP64
+// work (2 lane operations per SM and clock) on every SM (18 us with one entry
+// per thread of 128 and the operands read from global memory, m = 80).
+__global__ void __launch_bounds__(64) k_small_gemm(const double* __restrict__ A, int ta,
+                                                   const double* __restrict__ B, int tb,
+                                                   double* __restrict__ C, int m, double alpha,
+                                                   double gamma) {
+  __shared__ double sa[8][129], sb[8][129];  // rows of op(A), columns of op(B)
+  const int i0 = blockIdx.y * 8, j0 = blockIdx.x * 8;
+  for (int t = threadIdx.x; t < 8 * m; t += 64) {
+    // (consecutive threads along the operand's contiguous dimension)
+    const int ra = ta ? t % 8 : t / m, ka = ta ? t / 8 : t % m;
+    const int rb = tb ? t / m : t % 8, kb = tb ? t % m : t / 8;
+    sa[ra][ka] = i0 + ra < m ? (ta ? A[ka * m + i0 + ra] : A[(i0 + ra) * m + ka]) : 0.0;
+    sb[rb][kb] = j0 + rb < m ? (tb ? B[(j0 + rb) * m + kb] : B[kb * m + j0 + rb]) : 0.0;
   }
-  C[e] = alpha * acc + (i == j ? gamma : 0.0);
+  __syncthreads();
+  const int i = threadIdx.x >> 3, j = threadIdx.x & 7;
+  double acc = 0.0;
+#pragma unroll 4
+  for (int k = 0; k < m; ++k) acc = fma(sa[i][k], sb[j][k], acc);
+  if (i0 + i < m && j0 + j < m)
+    C[(i0 + i) * m + j0 + j] = alpha * acc + (i0 + i == j0 + j ? gamma : 0.0);
 }
 
 void small_gemm(const double* A, int ta, const double* B, int tb, double* C, int m, double alpha,
                 double gamma, cudaStream_t s) {
-  k_small_gemm<<<(m * m + 127) / 128, 128, 0, s>>>(A, ta, B, tb, C, m, alpha, gamma);
+  RF_CHECK(m >= 1 && m <= 128, RAFEAST_ERR_INVALID_ARG);
+  const dim3 grid((m + 7) / 8, (m + 7) / 8);
+  k_small_gemm<<<grid, 64, 0, s>>>(A, ta, B, tb, C, m, alpha, gamma);
   RF_LAUNCH();
 }
 
 template <typename T>
 static void jacobi_launch(const double* A, int m, double* w, double* V, T* Vg, int sweeps,
-                          double rot_tol, double off_tol, cudaStream_t s) {
+                          double rot_tol, double off_tol, double abs_tol, cudaStream_t s) {
   const int me = m + (m & 1);
   size_t smem = (size_t)me * me * sizeof(T);
   if (2 * smem <= JACOBI_SMEM_MAX) smem *= 2;  // V beside A
   ensure_dyn_smem(reinterpret_cast<const void*>(k_jacobi<T>), smem);
-  k_jacobi<T><<<1, 1024, smem, s>>>(A, m, w, V, Vg, sweeps, rot_tol, off_tol);
+  k_jacobi<T><<<1, 1024, smem, s>>>(A, m, w, V, Vg, sweeps, rot_tol, off_tol, abs_tol);
   RF_LAUNCH();
 }
 
+// U = I + E of a nearly diagonal symmetric B: the first-order rotations
+// e_ij = b_ij / (b_jj - b_ii) (Jacobi 1846; the separated case of Ogita and
+// Aishima, "Iterative refinement for symmetric eigenvalue decomposition", Japan
+// J. Indust. Appl. Math. 35, 2018). A pair with |e_ij| > 0.02 (a cluster) is
+// left to the Jacobi sweeps that follow, and so are all pairs of a row whose
+// |e_ij| add up to more than 0.1: ||E|| <= 0.1, and three Newton-Schulz steps
+// bring U^T U from I + 1e-2 to I + 2e-17. One CTA per row; full[i]: row i is
+// over the sum.
+__device__ __forceinline__ double first_order(const double* __restrict__ B, int m, int i, int j) {
+  if (i == j) return 0.0;
+  const double b = 0.5 * (B[i * m + j] + B[j * m + i]);
+  const double gap = B[j * m + j] - B[i * m + i];
+  return fabs(b) <= 0.02 * fabs(gap) && gap != 0.0 ? b / gap : 0.0;
+}
+__global__ void __launch_bounds__(128) k_first_order_sums(const double* __restrict__ B, int m,
+                                                          int* __restrict__ full) {
+  __shared__ double sw[4];
+  const int i = blockIdx.x;
+  const double e = threadIdx.x < m ? fabs(first_order(B, m, i, threadIdx.x)) : 0.0;
+  const double t = warp_sum(e);
+  if ((threadIdx.x & 31) == 0) sw[threadIdx.x >> 5] = t;
+  __syncthreads();
+  if (threadIdx.x == 0) full[i] = !(sw[0] + sw[1] + sw[2] + sw[3] <= 0.1);
+}
+__global__ void __launch_bounds__(128) k_first_order(const double* __restrict__ B, int m,
+                                                     const int* __restrict__ full,
+                                                     double* __restrict__ U) {
+  const int i = blockIdx.x, j = threadIdx.x;
+  if (j >= m) return;
+  U[i * m + j] = i == j ? 1.0 : (full[i] || full[j]) ? 0.0 : first_order(B, m, i, j);
+}
+
 // Mixed-precision Jacobi. GB300's FP64 rate is a small fraction of its FP32
-// rate, and a one-CTA Jacobi on an 80 x 80 matrix is bound by one SM's FP64
-// issue. So: (1) float Jacobi to the float rounding floor gives V1 with
-// V1^T A V1 diagonal to ~1e-7; (2) two Newton-Schulz steps
+// rate, and a one-CTA FP64 Jacobi sweep of an 80 x 80 matrix takes 0.8 ms of
+// one SM's FP64 issue. So: (1) float Jacobi to the float rounding floor gives
+// V1 with V1^T A V1 diagonal to ~1e-7; (2) two Newton-Schulz steps
 // V <- V (3 I - V^T V) / 2 make V1 orthonormal to working precision (its
-// float error is ~1e-6, each step squares it); (3) the FP64 Jacobi on
-// B = V^T A V, already nearly diagonal, needs a few sweeps; (4) V = V1 V_B.
-// The final accuracy is that of the FP64 Jacobi, as with FP64 alone.
+// float error is ~1e-6, each step squares it); (3) three rounds of first-order
+// rotations on B = V1^T A V1, U = I + E made orthonormal by three Newton-Schulz
+// steps, square its off-diagonal part for every pair that is not a cluster, by
+// products that run on all SMs; (4) FP64 Jacobi sweeps on what is left, none
+// when every entry is within a few units of rounding (8 eps of the root mean
+// square eigenvalue); (5) V = V1 U1 U2 U3 V_B. On the kNN Rayleigh-Ritz matrix of
+// 80 columns the FP64 part took 2.2 ms as Jacobi sweeps alone.
 void jacobi_eigh(double* A, int m, double* w, double* V, double* work, cudaStream_t s) {
   if (m > 128) throw Err{RAFEAST_ERR_INVALID_ARG};
   const int me = m + (m & 1);
@@ -695,7 +902,7 @@ void jacobi_eigh(double* A, int m, double* w, double* V, double* work, cudaStrea
   double* B = work + 3 * mm;
   double* VB = work + 4 * mm;
   double* Vg = work + 5 * mm;  // also the float stage's fallback accumulator
-  jacobi_launch<float>(A, m, w, W1, reinterpret_cast<float*>(Vg), 30, 1e-6, 1e-13, s);
+  jacobi_launch<float>(A, m, w, W1, reinterpret_cast<float*>(Vg), 30, 1e-6, 1e-13, 0.0, s);
   for (int it = 0; it < 2; ++it) {
     small_gemm(W1, 1, W1, 0, S, m, -0.5, 1.5, s);  // S = (3 I - V^T V) / 2
     small_gemm(W1, 0, S, 0, W2, m, 1.0, 0.0, s);   // V <- V S
@@ -703,51 +910,89 @@ void jacobi_eigh(double* A, int m, double* w, double* V, double* work, cudaStrea
   }
   small_gemm(A, 0, W1, 0, S, m, 1.0, 0.0, s);  // A V
   small_gemm(W1, 1, S, 0, B, m, 1.0, 0.0, s);  // V^T A V
-  jacobi_launch<double>(B, m, w, VB, Vg, 40, 1e-17, 1e-32, s);
+  for (int it = 0; it < 3; ++it) {
+    k_first_order_sums<<<m, 128, 0, s>>>(B, m, reinterpret_cast<int*>(S));
+    RF_LAUNCH();
+    k_first_order<<<m, 128, 0, s>>>(B, m, reinterpret_cast<const int*>(S), VB);
+    RF_LAUNCH();
+    for (int ns = 0; ns < 3; ++ns) {
+      small_gemm(VB, 1, VB, 0, S, m, -0.5, 1.5, s);  // (3 I - U^T U) / 2
+      small_gemm(VB, 0, S, 0, Vg, m, 1.0, 0.0, s);   // U
+      std::swap(VB, Vg);
+    }
+    small_gemm(B, 0, VB, 0, S, m, 1.0, 0.0, s);
+    small_gemm(VB, 1, S, 0, B, m, 1.0, 0.0, s);    // U^T B U
+    small_gemm(W1, 0, VB, 0, W2, m, 1.0, 0.0, s);  // V1 U
+    std::swap(W1, W2);
+  }
+  jacobi_launch<double>(B, m, w, VB, Vg, 40, 1e-17, 1e-32, 8 * DBL_EPSILON, s);
   small_gemm(W1, 0, VB, 0, V, m, 1.0, 0.0, s);  // V1 V_B
 }
 
 // ---------------------------------------------------------------------------
 // column reductions over rows
 // mode 0: out[i] = sum_r X[r][i] Y[r][i];  mode 1: out[i] = sum_r (Y - th_i X)^2
-// Block b sums the rows b, b + B, b + 2B, ... of every column into part[b];
-// a second kernel adds the B partial sums of each column in increasing b, so
+// Block b sums every B-th group of CR_G rows of every column into part[b];
+// a second kernel adds the B partial sums of each column in a fixed order, so
 // the result does not depend on the order in which blocks run.
 // ---------------------------------------------------------------------------
+constexpr int CR_G = 6;
 __global__ void k_colred(const double* __restrict__ X, const double* __restrict__ Y,
                          const double* __restrict__ th, int64_t n, int m, int ld, int mode,
                          double* part) {
+  // blockDim.y row groups of one thread per column, added in order at the end
+  __shared__ double sg[CR_G][128];
   const int i = threadIdx.x;
-  if (i >= m) return;
-  const double t = mode ? th[i] : 0.0;
+  const bool on = i < m;
+  const double t = mode && on ? th[i] : 0.0;
   double acc = 0.0;
-  for (int64_t r = blockIdx.x; r < n; r += gridDim.x) {
-    const double x = X[r * ld + i], y = Y[r * ld + i];
-    if (mode) {
-      const double d = y - t * x;
-      acc = fma(d, d, acc);
-    } else {
-      acc = fma(x, y, acc);
+  constexpr int U = 4;  // rows whose loads are in flight together
+  const int64_t step = (int64_t)gridDim.x * CR_G;
+  for (int64_t r0 = (int64_t)blockIdx.x * CR_G + threadIdx.y; on && r0 < n; r0 += U * step) {
+    double x[U], y[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t r = r0 + u * step;
+      x[u] = r < n ? X[r * ld + i] : 0.0;
+      y[u] = r < n ? Y[r * ld + i] : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (mode) {
+        const double d = y[u] - t * x[u];
+        acc = fma(d, d, acc);
+      } else {
+        acc = fma(x[u], y[u], acc);
+      }
     }
   }
-  part[(int64_t)blockIdx.x * m + i] = acc;
+  if (on) sg[threadIdx.y][i] = acc;
+  __syncthreads();
+  if (on && threadIdx.y == 0) {
+    for (int g = 1; g < CR_G; ++g) acc += sg[g][i];
+    part[(int64_t)blockIdx.x * m + i] = acc;
+  }
 }
 
-__global__ void k_colsum(const double* __restrict__ part, int nparts, int m, double* out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= m) return;
+// one warp per column: lane l adds the partials l, l + 32, ... in order, then
+// the lanes by a fixed tree
+__global__ void __launch_bounds__(32) k_colsum(const double* __restrict__ part, int nparts, int m,
+                                               double* out) {
+  const int i = blockIdx.x;
   double s = 0.0;
-  for (int b = 0; b < nparts; ++b) s += part[(int64_t)b * m + i];
-  out[i] = s;
+  for (int b = threadIdx.x; b < nparts; b += 32) s += part[(int64_t)b * m + i];
+  s = warp_sum(s);
+  if (threadIdx.x == 0) out[i] = s;
 }
 
 static void colred(const double* X, const double* Y, const double* th, int64_t n, int m, int ld,
                    int mode, double* out, double* part, int num_sms, cudaStream_t s) {
   const int threads = ((m + 31) / 32) * 32;
-  const int blocks = (int)std::min<int64_t>(n, 2 * (int64_t)num_sms);
-  k_colred<<<blocks, threads, 0, s>>>(X, Y, th, n, m, ld, mode, part);
+  RF_CHECK(m <= 128, RAFEAST_ERR_INVALID_ARG);
+  const int blocks = (int)std::min<int64_t>((n + CR_G - 1) / CR_G, 2 * (int64_t)num_sms);
+  k_colred<<<blocks, dim3(threads, CR_G), 0, s>>>(X, Y, th, n, m, ld, mode, part);
   RF_LAUNCH();
-  k_colsum<<<(m + 127) / 128, 128, 0, s>>>(part, blocks, m, out);
+  k_colsum<<<m, 32, 0, s>>>(part, blocks, m, out);
   RF_LAUNCH();
 }
 

@@ -1,0 +1,62 @@
+"""The m x m steps of the dense phase at the sizes where their kernels change:
+one warp, ragged blocks of eight, the largest width; layout moves on both
+sides of the small-block rule, reordered and not.
+
+Rayleigh-Ritz on a block whose Ritz values come in exact multiplicities (three
+equal grid sides) and on one with well separated values; tolerances are the
+backward errors of an m-column FP64 product, n u with u = 2^-53 and ||A||_1.
+"""
+import numpy as np
+import pytest
+
+from gpu_util import colmajor_dev, from_colmajor
+from workloads import graphs as G
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("m", [1, 2, 7, 33, 80, 127, 128])
+@pytest.mark.parametrize("kind", ["clusters", "random"])
+def test_rayleigh_ritz_is_a_decomposition(lib, m, kind):
+    import torch
+    lap = G.grid3d(11, 11, 11, 0.1)
+    A, n = lap.scipy(), lap.n
+    rng = np.random.default_rng(m)
+    if kind == "random":
+        q0 = np.linalg.qr(rng.standard_normal((n, m)))[0]
+    else:  # eigenvectors of the grid, rotated among themselves
+        import scipy.linalg as sl
+        v = sl.eigh(A.toarray(), subset_by_index=[0, m - 1])[1]
+        q0 = v @ np.linalg.qr(rng.standard_normal((m, m)))[0]
+    h = lib.rafeast_create(lap.row_ptr, lap.col_idx, lap.values, lap.shift)
+    try:
+        Q = colmajor_dev(q0)
+        theta, _ = lib.rafeast_rayleigh_ritz(h, m, Q)
+        q = from_colmajor(Q)
+        tol = n * 2.0 ** -53 * 12.1
+        assert np.all(np.diff(theta) >= 0)
+        assert np.abs(q.T @ q - np.eye(m)).max() <= tol
+        assert np.abs(q.T @ (A @ q) - np.diag(theta)).max() <= tol
+        assert np.linalg.norm(q - q0 @ (q0.T @ q)) <= tol * m
+        R = lib.rafeast_orthonormalize(h, m, colmajor_dev(q0 * np.logspace(0, -3, m)), want_r=True)
+        assert np.allclose(np.abs(np.diag(R)), np.logspace(0, -3, m), rtol=tol)
+    finally:
+        lib.rafeast_destroy(h)
+
+
+@pytest.mark.parametrize("n,k", [(31, 3), (33, 130), (8191, 64), (8193, 65), (20011, 27)])
+@pytest.mark.parametrize("flag", [1, 2])  # the caller's row order, a reordering
+def test_layout_moves_keep_every_entry(lib, n, k, flag):
+    """A x for integer-valued x is exact in FP64, so the product shows that each
+    entry went to its place and came back."""
+    import torch
+    lap = G.cycle(n, 1.0) if hasattr(G, "cycle") else G.grid2d(n, 1, 1.0)
+    x = np.arange(n * k, dtype=np.float64).reshape(n, k) % 1021
+    h = lib.rafeast_create(lap.row_ptr, lap.col_idx, lap.values, lap.shift, flags=flag)
+    try:
+        X = colmajor_dev(x)
+        Y = torch.full_like(X, -1.0)
+        lib.rafeast_spmm(h, k, 1.0, 0.0, X, Y)
+        assert np.array_equal(from_colmajor(Y), lap.scipy() @ x)
+    finally:
+        lib.rafeast_destroy(h)
