@@ -1757,6 +1757,269 @@ static void filter_ms_batched(std::vector<BatchItem*>& items, Handle* owner, cud
   for (auto* it : items) RF_CUDA(cudaStreamWaitEvent(it->h->stream, owner->ev_in, 0));
 }
 
+// the Lanczos form of the batched filter: grouped products and updates for all
+// problems in lockstep steps, then every problem's collapse and combine on its
+// own stream
+template <typename T>
+static void filter_lz_batched(std::vector<BatchItem*>& items, Handle* owner, cudaStream_t bs,
+                              int64_t sig, bool tight) {
+  const int cnt = (int)items.size();
+  if (cnt == 0) return;
+  const bool fp64 = sizeof(T) == 8, prof = owner->opt_profile != 0;
+  for (auto* it : items) {  // every problem's inputs were produced on its own stream
+    RF_CUDA(cudaEventRecord(it->h->ev_out, it->h->stream));
+    RF_CUDA(cudaStreamWaitEvent(bs, it->h->ev_out, 0));
+  }
+  size_t off = 0;
+  auto carve = [&](size_t bytes) {
+    off = (off + 255) & ~(size_t)255;
+    size_t o = off;
+    off += bytes;
+    return o;
+  };
+  const size_t o_ctl = carve(sizeof(CocgCtl) * cnt);
+  const size_t o_args = carve(sizeof(LzArgs<T>) * cnt);
+  const size_t o_md = carve(sizeof(int) * (2 * cnt + 1));
+  const size_t o_mu = carve(sizeof(int) * (2 * cnt + 1));
+  const size_t o_gc = carve(sizeof(GroupCtl));
+  const size_t o_ggd = carve(sizeof(int) * 4 * cnt);
+  const size_t o_ggu = carve(sizeof(int) * 4 * cnt);
+  char* bb = (char*)scratch(owner, S_BATCH, off + 256);
+  CocgCtl* ctl_d = (CocgCtl*)(bb + o_ctl);
+  std::vector<LzProblem<T>> P(cnt);
+  bool all_vf = true;
+  double cells = 0.0;
+  int max_inner = 1;
+  for (int t = 0; t < cnt; ++t) {
+    Handle* h = items[t]->h;
+    // (replays are as long as the first handle asks)
+    const int chunk = h->opt_chunk;
+    h->opt_chunk = owner->opt_chunk;
+    try {
+      P[t] = lz_setup<T>(h, *items[t]->prm, h->Q, h->AQ, h->theta_d, h->theta, h->m0, h->ldq,
+                         ctl_d + t, prof, tight, bs);
+    } catch (...) {
+      h->opt_chunk = chunk;
+      throw;
+    }
+    h->opt_chunk = chunk;
+    all_vf = all_vf && P[t].a.lcolidx != nullptr;
+    cells += (double)P[t].a.stride;
+    max_inner = std::max(max_inner, items[t]->prm->max_inner);
+  }
+  if (!owner->mem_total) {
+    size_t mem_free = 0;
+    RF_CUDA(cudaMemGetInfo(&mem_free, &owner->mem_total));
+  }
+  LzGroupDev<T> gd;
+  gd.args = (const LzArgs<T>*)(bb + o_args);
+  gd.map_d = (int*)(bb + o_md);
+  gd.map_u = (int*)(bb + o_mu);
+  gd.gc = (GroupCtl*)(bb + o_gc);
+  gd.ctl = ctl_d;
+  gd.gg_d = (const int4*)(bb + o_ggd);
+  gd.gg_u = (const int4*)(bb + o_ggu);
+  GroupPlan plan;
+  std::vector<LzArgs<T>> args(cnt);
+  // the product's shape (lanes, chunks; 0: each problem's own default); the
+  // device has finished every earlier replay
+  auto prepare = [&](int G, int cpl, int dry) {
+    for (int t = 0; t < cnt; ++t) {
+      LzArgs<T>& a = args[t];
+      a = P[t].a;
+      if (!all_vf) {  // values-free gathers only when every problem has them
+        a.lrowptr = nullptr;
+        a.lcolidx = nullptr;
+      }
+      if (G) {
+        a.lanes = G;
+        a.cpl = cpl;
+      }
+      a.dry = dry;
+    }
+    plan = GroupPlan();
+    plan_lz_grouped<T>(args, owner->num_sms, plan);
+    GroupCtl gch;
+    memset(&gch, 0, sizeof(gch));
+    gch.grid_d = plan.ctas_dots;
+    gch.grid_u = plan.ctas_upd;
+    auto up = [&](size_t o, const void* p, size_t bytes) {
+      RF_CUDA(cudaMemcpyAsync(bb + o, p, bytes, cudaMemcpyHostToDevice, bs));
+    };
+    up(o_args, args.data(), sizeof(LzArgs<T>) * cnt);
+    up(o_md, plan.map_dots.data(), sizeof(int) * plan.map_dots.size());
+    up(o_mu, plan.map_upd.data(), sizeof(int) * plan.map_upd.size());
+    up(o_gc, &gch, sizeof(gch));
+    up(o_ggd, plan.gg_d.data(), sizeof(int) * plan.gg_d.size());
+    up(o_ggu, plan.gg_u.data(), sizeof(int) * plan.gg_u.size());
+    RF_CUDA(cudaStreamSynchronize(bs));  // (the host copies go out of scope or change)
+  };
+  // autotuner of the product's shape for the whole batch (as filter_lz_run's),
+  // kept under the batch's signature on the first handle
+  const int64_t key = sig ^ ((int64_t)1 << 61);
+  Handle::Shape shp{0, 0, 0, 0};
+  bool have = false;
+  for (auto& kv : owner->tuned)
+    if (kv.first == key) {
+      shp = kv.second;
+      have = true;
+    }
+  if (!have && owner->opt_autotune) {
+    const int cand[][2] = {{0, 0}, {16, 1}, {8, 1}, {8, 2}, {4, 1}, {4, 2}, {16, 2}};
+    float best = 1e30f;
+    cudaEvent_t ev[3];
+    for (auto& e : ev) RF_CUDA(cudaEventCreate(&e));
+    for (auto& c : cand) {
+      prepare(c[0], c[1], 1);
+      for (int r = 0; r < 2; ++r) {
+        RF_CUDA(cudaEventRecord(ev[r], bs));
+        launch_lz_grouped<T>(plan, gd, 0, bs);
+      }
+      RF_CUDA(cudaEventRecord(ev[2], bs));
+      RF_CUDA(cudaStreamSynchronize(bs));
+      owner->launches += 2;
+      float ms = 0.f;
+      RF_CUDA(cudaEventElapsedTime(&ms, ev[1], ev[2]));
+      if (ms < best) {
+        best = ms;
+        shp.dl = c[0];
+        shp.dc = c[1];
+      }
+    }
+    for (auto& e : ev) RF_CUDA(cudaEventDestroy(e));
+    owner->tuned.push_back(std::make_pair(key, shp));
+  }
+  prepare(shp.dl, shp.dc, 0);
+  owner->prof[6] = shp.dl * 100 + shp.dc;
+  owner->prof[7] = P[0].a.sl;
+  const int steps = lz_replay_steps(owner, tight);
+  std::vector<cudaEvent_t> evs;
+  if (prof) {
+    evs.resize(2 * steps + 1);
+    for (auto& e : evs) RF_CUDA(cudaEventCreate(&e));
+  }
+  struct ExecGuard {
+    cudaGraphExec_t exec = nullptr;
+    ~ExecGuard() {
+      if (exec) cudaGraphExecDestroy(exec);
+    }
+  } guard;
+  cudaGraph_t graph = nullptr;
+  RF_CUDA(cudaStreamBeginCapture(bs, cudaStreamCaptureModeThreadLocal));
+  g_capturing = true;
+  try {
+    for (int it = 0; it < steps; ++it) {
+      if (prof) RF_CUDA(cudaEventRecordWithFlags(evs[2 * it], bs, cudaEventRecordExternal));
+      launch_lz_grouped<T>(plan, gd, 0, bs);
+      if (prof) RF_CUDA(cudaEventRecordWithFlags(evs[2 * it + 1], bs, cudaEventRecordExternal));
+      launch_lz_grouped<T>(plan, gd, 1, bs);
+    }
+    if (prof) RF_CUDA(cudaEventRecordWithFlags(evs[2 * steps], bs, cudaEventRecordExternal));
+  } catch (...) {
+    g_capturing = false;
+    cudaStreamEndCapture(bs, &graph);
+    if (graph) cudaGraphDestroy(graph);
+    throw;
+  }
+  g_capturing = false;
+  RF_CUDA(cudaStreamEndCapture(bs, &graph));
+  RF_CUDA(cudaGraphInstantiate(&guard.exec, graph, 0));
+  RF_CUDA(cudaGraphDestroy(graph));
+  std::vector<CocgCtl> ctl(cnt);
+  for (auto& c : ctl) memset(&c, 0, sizeof(c));
+  std::vector<int> k0(cnt, 0), cap(cnt);
+  std::vector<char> wrapped(cnt, 0);
+  for (int t = 0; t < cnt; ++t) cap[t] = (int)items[t]->h->lz_slabs.size() * P[t].a.sl;
+  std::vector<float> tk;
+  bool all_done = false;
+  const int max_replays = (max_inner + 2) / steps + 2;
+  for (int r = 0; r < max_replays && !all_done; ++r) {
+    for (int t = 0; t < cnt; ++t) {
+      if (ctl[t].done) continue;
+      Handle* h = items[t]->h;
+      const int k = ctl[t].iter;
+      if (k - k0[t] + steps + 1 > cap[t] && !wrapped[t]) {
+        // a batch's rings share a quarter of the device's memory by size
+        const size_t budget =
+            tight ? 0 : (size_t)(owner->mem_total / 4 * ((double)P[t].a.stride / cells));
+        const int got = lz_grow(h, P[t].a.stride, P[t].a.sl, 0, (int64_t)k + steps + 1, budget);
+        if (got != cap[t]) {
+          cap[t] = got;
+          lz_ring_upload(h, P[t].a, bs);
+        }
+      }
+      if (k - k0[t] + steps + 1 > cap[t]) {
+        wrapped[t] = 1;
+        lz_collapse<T>(h, P[t].a, k0[t], k, false, bs);
+        k0[t] = k;
+      }
+    }
+    RF_CUDA(cudaGraphLaunch(guard.exec, bs));
+    RF_CUDA(cudaMemcpyAsync(ctl.data(), ctl_d, sizeof(CocgCtl) * cnt, cudaMemcpyDeviceToHost, bs));
+    RF_CUDA(cudaStreamSynchronize(bs));
+    if (prof)
+      for (int q = 0; q < 2 * steps; ++q) {
+        float ms = 0.f;
+        RF_CUDA(cudaEventElapsedTime(&ms, evs[q], evs[q + 1]));
+        tk.push_back(ms);
+      }
+    owner->launches += 2 * steps;
+    owner->spmm_launches += steps;
+    all_done = true;
+    for (int t = 0; t < cnt; ++t) all_done = all_done && ctl[t].done;
+  }
+  for (auto& e : evs) RF_CUDA(cudaEventDestroy(e));
+  if (prof && all_done) {
+    int nsteps = 0;
+    std::vector<std::vector<int>> hist(cnt);
+    for (int t = 0; t < cnt; ++t) {
+      const int iters = std::min(ctl[t].iter, items[t]->prm->max_inner + 1);
+      hist[t].assign(iters, 0);
+      if (iters > 0 && P[t].a.hist)
+        RF_CUDA(cudaMemcpy(hist[t].data(), P[t].a.hist, sizeof(int) * iters,
+                           cudaMemcpyDeviceToHost));
+      nsteps = std::max(nsteps, iters);
+    }
+    for (int k = 0; k < nsteps && 2 * k + 1 < (int)tk.size(); ++k) {
+      double bd = 0.0, bu = 0.0;
+      int probs = 0, cols = 0;
+      for (int t = 0; t < cnt; ++t) {
+        if (k >= (int)hist[t].size()) continue;
+        const int act = k == 0 ? P[t].m0 : hist[t][k - 1];
+        bd += lz_dots_bytes(items[t]->h, act, fp64, all_vf);
+        if (hist[t][k] > 0) bu += lz_update_bytes(items[t]->h, hist[t][k], k, fp64);
+        probs += act > 0;
+        cols += act;
+      }
+      owner->last_hist.push_back(cols);
+      owner->last_rhist.push_back((double)probs);
+      owner->last_tk.push_back(tk[2 * k]);
+      owner->last_tk.push_back(tk[2 * k + 1]);
+      owner->prof[0] += 1;
+      owner->prof[1] += tk[2 * k];
+      owner->prof[2] += bd;
+      if (bu > 0.0) {
+        owner->prof[3] += 1;
+        owner->prof[4] += tk[2 * k + 1];
+        owner->prof[5] += bu;
+      }
+    }
+  }
+  // every problem goes on on its own stream: its collapse is a latency chain
+  // over the steps, and the problems' chains overlap
+  RF_CUDA(cudaEventRecord(owner->ev_in, bs));
+  for (int t = 0; t < cnt; ++t) {
+    Handle* h = items[t]->h;
+    RF_CUDA(cudaStreamWaitEvent(h->stream, owner->ev_in, 0));
+    try {
+      if (ctl[t].done) lz_collapse<T>(h, P[t].a, k0[t], ctl[t].iter, true, h->stream);
+      lz_finish_filter<T>(h, P[t], h->Q, h->ldq, items[t]->Qt, ctl[t], items[t]->fs, h->stream);
+    } catch (const Err& e) {
+      items[t]->err = e.code;
+    }
+  }
+}
+
 static void validate_params(const rafeast_params* p) {
   RF_CHECK(p, RAFEAST_ERR_INVALID_ARG);
   RF_CHECK(std::isfinite(p->lmin) && std::isfinite(p->lmax) && p->lmin < p->lmax,
@@ -3118,8 +3381,26 @@ int rafeast_solve_batched(int count, rafeast_t const* hs, const rafeast_params* 
         RF_CUDA(cudaEventRecord(runs[t].ev[2], bs));
       }
     if (act.empty()) break;
-    if (prms[0].precision == RAFEAST_FP64) filter_ms_batched<double>(act_items, owner, bs, sig);
-    else filter_ms_batched<float>(act_items, owner, bs, sig);
+    const bool fp64 = prms[0].precision == RAFEAST_FP64;
+    if (owner->opt_update == 0) {
+      auto run = [&](bool tight) {
+        if (fp64) filter_lz_batched<double>(act_items, owner, bs, sig, tight);
+        else filter_lz_batched<float>(act_items, owner, bs, sig, tight);
+      };
+      try {
+        run(false);
+      } catch (const Err& e) {  // (memory: once more with the smallest rings)
+        if (e.code != RAFEAST_ERR_OUT_OF_MEMORY) throw;
+        RF_CUDA(cudaDeviceSynchronize());
+        for (auto* i : act_items) lz_free(i->h);
+        clear_last_error();
+        run(true);
+      }
+    } else if (fp64) {
+      filter_ms_batched<double>(act_items, owner, bs, sig);
+    } else {
+      filter_ms_batched<float>(act_items, owner, bs, sig);
+    }
     for (int t : act) {
       runs[t].fs = items[t].fs;
       runs[t].cocg_total += items[t].fs.iters_max;

@@ -473,6 +473,21 @@ template <typename T> struct GroupDev {
   const int4* gg_d;
   const int4* gg_u;
 };
+// the Lanczos form's grouped kernels: args with one shape of the product
+template <typename T> struct LzGroupDev {
+  const LzArgs<T>* args;
+  int* map_d;
+  int* map_u;
+  GroupCtl* gc;
+  const CocgCtl* ctl;
+  const int4* gg_d;
+  const int4* gg_u;
+};
+template <typename T>
+void plan_lz_grouped(const std::vector<LzArgs<T>>& args, int num_sms, GroupPlan& g);
+template <typename T>
+void launch_lz_grouped(const GroupPlan& g, const LzGroupDev<T>& d, int which, cudaStream_t s);
+
 template <typename T>
 void plan_ms_grouped(const std::vector<CocgArgs<T>>& args_d, const std::vector<CocgArgs<T>>& args_u,
                      int num_sms, GroupPlan& g);

@@ -22,6 +22,7 @@
 #include <cstdio>
 
 #include "cocg_kernels.cuh"
+#include "lanczos.cuh"
 
 namespace rafeast {
 
@@ -263,6 +264,68 @@ __global__ void __launch_bounds__(THREADS)
   }
 }
 
+// ---- the Lanczos form (lanczos.cuh) over the same queues ----------------------
+// A problem's `done` is set by the update, so the maps planned at the end of a
+// product still hold a problem that the update after it finishes; its items
+// then return at once.
+template <typename T, int MAXCPL, bool VF>
+__global__ void __launch_bounds__(THREADS, MAXCPL == 1 ? 4 : MAXCPL == 2 ? 3 : 2)
+    k_lz_dots_grouped(const LzArgs<T>* __restrict__ args, int* __restrict__ map_d,
+                      int* __restrict__ map_u, GroupCtl* __restrict__ gc,
+                      const CocgCtl* __restrict__ ctl, const int4* __restrict__ gg_d,
+                      const int4* __restrict__ gg_u, int count) {
+  __shared__ int smap[2 * SMEM_MAP + 1];
+  __shared__ int s_glast;
+  const MapView m = stage_map(map_d, count, smap);
+  const int total = m[count];
+  for (;;) {
+    const int item = next_item(&gc->next_d, total);
+    if (item < 0) break;
+    const int t = item_owner(m, count, item);
+    const LzArgs<T> a = args[t];
+    lz_dots_body<T, MAXCPL, VF>(a, item_blk(m, count, t, item));
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_glast = atomicAdd(&gc->ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (s_glast) {
+    __threadfence();
+    plan_items(ctl, gg_d, gg_u, count, gc->grid_d, gc->grid_u, map_d, map_u);
+    if (threadIdx.x == 0) {
+      gc->next_d = 0;
+      gc->next_u = 0;
+      gc->ticket = 0;
+      __threadfence();
+    }
+  }
+}
+
+// an item: a range of one problem's rows and its share of the problem's scalars
+template <typename T>
+__global__ void __launch_bounds__(THREADS)
+    k_lz_update_grouped(const LzArgs<T>* __restrict__ args, const int* __restrict__ map,
+                        GroupCtl* __restrict__ gc, int count) {
+  __shared__ int smap[2 * SMEM_MAP + 1];
+  const MapView m = stage_map(map, count, smap);
+  const int total = m[count];
+  for (;;) {
+    const int item = next_item(&gc->next_u, total);
+    if (item < 0) break;
+    const int t = item_owner(m, count, item);
+    const LzArgs<T> a = args[t];
+    // (an item with a share of the scalars cannot see `done` set by this step:
+    // it waits for every share; the others have no barrier below)
+    if (__ldcg(&a.ctl->done)) continue;
+    const Blk b = item_blk(m, count, t, item);
+    lz_scalar_share<T>(a, __ldcg(&a.dyn->k) - 1, b.x, min(b.gx, a.ld));
+    const int64_t per = (a.n + b.gx - 1) / b.gx, r0 = b.x * per;
+    if (r0 < a.n) lz_update_rows<T>(a, r0, r0 + per < a.n ? r0 + per : a.n);
+  }
+}
+
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
@@ -448,6 +511,82 @@ void launch_ms_grouped(const GroupPlan& g, const GroupDev<T>& d, int which, int 
   }
   RF_LAUNCH();
 }
+
+template <typename T, int MC>
+static const void* lz_dots_fn(bool vf) {
+  return vf ? reinterpret_cast<const void*>(k_lz_dots_grouped<T, MC, true>)
+            : reinterpret_cast<const void*>(k_lz_dots_grouped<T, MC, false>);
+}
+
+template <typename T>
+void plan_lz_grouped(const std::vector<LzArgs<T>>& args, int num_sms, GroupPlan& g) {
+  const int cnt = (int)args.size();
+  RF_CHECK(cnt >= 1, RAFEAST_ERR_INVALID_ARG);
+  g.count = cnt;
+  int cd = 1, ln = 4, ld = 4;
+  const bool vf = args[0].lcolidx != nullptr;
+  for (const auto& a : args) {
+    RF_CHECK(a.cpl >= 1 && a.cpl <= 4 && a.nq <= THREADS && (a.lcolidx != nullptr) == vf,
+             RAFEAST_ERR_INVALID_ARG);
+    cd = std::max(cd, a.cpl);
+    ln = std::max(ln, a.lanes);
+    ld = std::max(ld, a.ld);
+  }
+  const int mc = cd == 1 ? 1 : cd == 2 ? 2 : 4;
+  g.mc_d = mc;
+  g.fn_dots = mc == 1 ? lz_dots_fn<T, 1>(vf) : mc == 2 ? lz_dots_fn<T, 2>(vf) : lz_dots_fn<T, 4>(vf);
+  g.fn_upd = reinterpret_cast<const void*>(k_lz_update_grouped<T>);
+  g.smem_dots = lz_dots_smem<T>(ln, mc, ld);
+  g.smem_upd = 0;
+  if (g.smem_dots > 48 * 1024) ensure_dyn_smem(g.fn_dots, g.smem_dots);
+  int occ_d = 0, occ_u = 0;
+  RF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_d, g.fn_dots, THREADS, g.smem_dots));
+  RF_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_u, g.fn_upd, THREADS, 0));
+  g.gg_d.assign(4 * cnt, 0);
+  g.gg_u.assign(4 * cnt, 0);
+  long long wkb = 0;
+  for (int t = 0; t < cnt; ++t) {
+    const auto& a = args[t];
+    const int64_t per = (int64_t)WARPS * (32 / a.lanes), peru = THREADS / a.nq;
+    const int64_t gd = (a.n + per - 1) / per, gu = (a.n + peru - 1) / peru;
+    RF_CHECK(gd < 0x7fffffff && gu < 0x7fffffff, RAFEAST_ERR_INVALID_ARG);
+    g.gg_d[4 * t] = (int)gd;
+    g.gg_d[4 * t + 1] = (a.nq + a.lanes * a.cpl - 1) / (a.lanes * a.cpl);
+    // the gathered vector (the CTAs in flight share about WINDOW_KB of it)
+    g.gg_d[4 * t + 2] = (int)std::min<int64_t>(
+        0x7fffffff, (a.n * (int64_t)a.ld * (int64_t)sizeof(T) + 1023) / 1024);
+    g.gg_u[4 * t] = (int)gu;
+    g.gg_u[4 * t + 1] = 1;
+    wkb += g.gg_d[4 * t + 2];
+  }
+  g.ctas_dots = num_sms * std::max(occ_d, 1);
+  g.ctas_upd = num_sms * std::max(occ_u, 1);
+  plan_host(g.gg_d, wkb, g.ctas_dots, g.map_dots);
+  plan_host(g.gg_u, wkb, g.ctas_upd, g.map_upd);
+}
+
+template <typename T>
+void launch_lz_grouped(const GroupPlan& g, const LzGroupDev<T>& d, int which, cudaStream_t s) {
+  int cnt = g.count;
+  GroupCtl* gc = d.gc;
+  const LzArgs<T>* ap = d.args;
+  int *md = d.map_d, *mu = d.map_u;
+  if (which == 0) {
+    const CocgCtl* ctl = d.ctl;
+    const int4 *ggd = d.gg_d, *ggu = d.gg_u;
+    void* params[] = {(void*)&ap,  (void*)&md,  (void*)&mu,  (void*)&gc,
+                      (void*)&ctl, (void*)&ggd, (void*)&ggu, (void*)&cnt};
+    RF_CUDA(cudaLaunchKernel(g.fn_dots, dim3(g.ctas_dots), dim3(THREADS), params, g.smem_dots, s));
+  } else {
+    void* params[] = {(void*)&ap, (void*)&mu, (void*)&gc, (void*)&cnt};
+    RF_CUDA(cudaLaunchKernel(g.fn_upd, dim3(g.ctas_upd), dim3(THREADS), params, 0, s));
+  }
+  RF_LAUNCH();
+}
+template void plan_lz_grouped<float>(const std::vector<LzArgs<float>>&, int, GroupPlan&);
+template void plan_lz_grouped<double>(const std::vector<LzArgs<double>>&, int, GroupPlan&);
+template void launch_lz_grouped<float>(const GroupPlan&, const LzGroupDev<float>&, int, cudaStream_t);
+template void launch_lz_grouped<double>(const GroupPlan&, const LzGroupDev<double>&, int, cudaStream_t);
 
 template void plan_ms_grouped<float>(const std::vector<CocgArgs<float>>&,
                                      const std::vector<CocgArgs<float>>&, int, GroupPlan&);

@@ -63,6 +63,8 @@ __global__ void __launch_bounds__(THREADS, MINB) k_lz_dots(LzArgs<T> a) {
 
 template <typename T>
 __global__ void __launch_bounds__(THREADS) k_lz_update(LzArgs<T> a) {
+  // (a CTA with a share of the scalars cannot see `done` set by this step: it
+  // waits for every share; the others have no barrier below)
   if (__ldcg(&a.ctl->done)) return;
   lz_scalar_share<T>(a, __ldcg(&a.dyn->k) - 1, blockIdx.x, min((int)gridDim.x, a.ld));
   // contiguous row ranges, CTA 0 at the top

@@ -205,39 +205,52 @@ __device__ __forceinline__ void lz_nodes(const LzArgs<T>& a, int k, int c, doubl
   }
 }
 
-// the scalar share of CTA b of nb: columns b, b + nb, ... (warp 0; every CTA
-// with a share calls it, nb <= ld); the last of them ends the step
+// the scalar share of CTA b of nb: warp w takes the columns b + nb w,
+// + 8 nb, ...; every CTA with a share (b < nb <= ld) calls it with all its
+// threads. The last of them ends the step.
 template <typename T>
 __device__ __forceinline__ void lz_scalar_share(const LzArgs<T>& a, int k, int b, int nb) {
-  if (threadIdx.x >= 32 || b >= nb) return;
+  if (b >= nb) return;
   constexpr int V = LZV<T>;
+  __shared__ MsCount sc[WARPS];
+  __shared__ int s_end;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   MsCount cnt;
   ms_count_init(cnt);
   double2* th = lz_th(a, (char*)__ldcg((const unsigned long long*)&a.dyn->uu));
-  for (int c = b; c < a.ld; c += nb) lz_nodes<T>(a, k, c, th, cnt);
+  for (int c = b + nb * warp; c < a.ld; c += nb * WARPS) lz_nodes<T>(a, k, c, th, cnt);
+  if (lane == 0) sc[warp] = cnt;
+  __syncthreads();
   CocgCtl* ctl = a.ctl;
-  int last = 0;
   if (threadIdx.x == 0) {
+    for (int w = 1; w < WARPS; ++w) {
+      cnt.active += sc[w].active;
+      cnt.brk += sc[w].brk;
+      cnt.cap += sc[w].cap;
+      cnt.mx = max(cnt.mx, sc[w].mx);
+      cnt.mn = min(cnt.mn, sc[w].mn);
+      cnt.worst = fmax(cnt.worst, sc[w].worst);
+    }
     if (cnt.active) atomicAdd(&ctl->g_active, cnt.active);
     if (cnt.brk) atomicAdd(&ctl->g_brk, cnt.brk);
     if (cnt.cap) atomicAdd(&ctl->g_cap, cnt.cap);
     if (cnt.mx) atomicMax(&ctl->g_mx, cnt.mx);
     if (cnt.mn != 0x7fffffff) atomicMin(&ctl->g_mn, cnt.mn);
     if (a.hist) atomicMax(&ctl->g_worst, (unsigned long long)__double_as_longlong(cnt.worst));
+    __threadfence();
+    s_end = atomicAdd(&ctl->ticket2, 1u) == (unsigned)nb - 1;
   }
+  __syncthreads();
+  if (!s_end || warp != 0) return;
   __threadfence();
-  __syncwarp();
-  if (threadIdx.x == 0) last = atomicAdd(&ctl->ticket2, 1u) == (unsigned)nb - 1;
-  if (!__shfl_sync(0xffffffffu, last, 0)) return;
-  __threadfence();
-  for (int q = threadIdx.x; q < a.nq; q += 32) {
+  for (int q = lane; q < a.nq; q += 32) {
     int any = 0;
 #pragma unroll
     for (int v = 0; v < V; ++v) any |= __ldcg(&a.col[q * V + v].kstop) == LZ_RUNS;
     a.qact[q] = any;
   }
   __syncwarp();
-  if (threadIdx.x == 0) {
+  if (lane == 0) {
     const int act = __ldcg(&ctl->g_active), mx = __ldcg(&ctl->g_mx), mn = __ldcg(&ctl->g_mn);
     if (a.hist && k <= a.max_inner) {
       a.hist[k] = act;

@@ -77,3 +77,32 @@ def test_zero_column_and_nan_input(lib):
             assert ei.value.code == lib.RAFEAST_ERR_COCG_BREAKDOWN
     finally:
         lib.rafeast_destroy(h)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_batched_filter_matches_one_at_a_time(lib, prec):
+    """Two outer iterations of a batch of uneven grids (one row block to many;
+    problems that stop at different steps) against rafeast_solve on the same
+    start: the grouped launches change only the order of the sums."""
+    shapes, m0s = [(5, 7), (20, 23), (37, 41), (90, 101)], [3, 8, 17, 30]
+    p = lib.RAFEAST_FP64 if prec == "fp64" else lib.RAFEAST_MIXED
+    laps = [G.grid2d(a, b, shift=0.1 * (t + 1)) for t, (a, b) in enumerate(shapes)]
+    prms = [lib.make_params(0.05, 0.1 * (t + 1) + 0.3, m, 3, 0.5, 1e-3, 0.0, 2, 40 + 13 * t, p,
+                            lib.RAFEAST_FORM_CORRECTION, lib.RAFEAST_START_RANDOM, 5)
+            for t, m in enumerate(m0s)]
+    hs = [lib.rafeast_create(x.row_ptr, x.col_idx, x.values, x.shift) for x in laps]
+    h1 = [lib.rafeast_create(x.row_ptr, x.col_idx, x.values, x.shift) for x in laps]
+    try:
+        ev = [np.zeros(m) for m in m0s]
+        _, mf, _ = lib.rafeast_solve_batched(hs, prms, ev)
+        for t, m in enumerate(m0s):
+            e1 = np.zeros(m)
+            _, mf1, _ = lib.rafeast_solve(h1[t], prms[t], e1)
+            assert mf1 == mf[t]
+            # Ritz values after two filters: errors enter squared; 2^9 units of
+            # the working precision of the filter, relative to ||A||_1 < 8.5
+            eps = 2.0 ** -52 if prec == "fp64" else 2.0 ** -23
+            assert np.max(np.abs(np.sort(ev[t]) - np.sort(e1))) <= 2.0 ** 9 * eps * 8.5
+    finally:
+        for h in hs + h1:
+            lib.rafeast_destroy(h)
