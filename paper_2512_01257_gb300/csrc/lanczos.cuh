@@ -197,7 +197,7 @@ __device__ __forceinline__ void lz_nodes(const LzArgs<T>& a, int k, int c, doubl
     if (any) {
       o.s = s;
       o.is = is;
-      o.sq = sqrt(st.bnorm2 * st.rr);
+      o.sq = sqrt(st.bnorm2) * sqrt(st.rr);  // (their product may leave the range)
       ++cnt.active;
     } else {
       o.kstop = k;

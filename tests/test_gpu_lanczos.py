@@ -106,3 +106,31 @@ def test_batched_filter_matches_one_at_a_time(lib, prec):
     finally:
         for h in hs + h1:
             lib.rafeast_destroy(h)
+
+
+def test_columns_of_extreme_norm(lib):
+    """The filter is linear: FP64 columns times 2^-332 and 2^332 (squared norms
+    within the double range, their products not) give the same results times
+    that. Scaling by powers of two rounds nothing, so the two results differ by
+    the order of the sums alone: 2^9 eps of test_fixed_steps_match_oracle's
+    bound each."""
+    import torch
+    lap = G.grid2d(37, 41, shift=0.3)
+    q0 = OF.random_start(lap.n, 6, 3)
+    scale = np.array([1.0, 2.0 ** -332, 2.0 ** 332])
+    z, w = OQ.nodes(0.31, 0.6, 2, 1.0)
+    bound = 2.0 ** 10 * 2.0 ** -52 * OF.one_norm(lap.scipy()) * np.sum(np.abs(w) / z.imag ** 2)
+    h = lib.rafeast_create(lap.row_ptr, lap.col_idx, lap.values, lap.shift)
+    try:
+        out = []
+        for x in scale:
+            prm = lib.make_params(0.31, 0.6, 6, 2, 1.0, 0.0, 1e-10, 1, 40, lib.RAFEAST_FP64,
+                                  lib.RAFEAST_FORM_DIRECT)
+            Q = colmajor_dev(q0 * x)
+            Qt = torch.zeros_like(Q)
+            lib.rafeast_filter(h, prm, Q, None, Qt)
+            out.append(from_colmajor(Qt) / x)
+        for y in out[1:]:
+            assert np.max(np.linalg.norm(y - out[0], axis=0)) <= bound
+    finally:
+        lib.rafeast_destroy(h)
