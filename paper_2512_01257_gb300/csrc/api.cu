@@ -1057,11 +1057,21 @@ struct LzProblem {
 // Slots are allocated as a solve needs them, up to a share of the device's
 // memory (LZ_RING_SHARE); a solve with more steps than slots folds full rings
 // into its directions. A slab is about a gigabyte or the whole of 32 slots.
+// All handles' rings on a device together grow to a quarter of its memory at
+// most (beyond the slots a replay cannot do without), so that many handles
+// kept side by side leave room for the program's own tensors.
 constexpr size_t LZ_RING_SHARE = 16;  // a sixteenth of the device's memory
-static void lz_free(Handle* h) {
+constexpr size_t LZ_RINGS_SHARE = 4;  // all rings
+static std::atomic<long long> g_ring_bytes[64];  // by device (a larger index: not bounded)
+static void lz_ring_drop(Handle* h) {
   for (void* p : h->lz_slabs) cudaFree(p);
+  if (h->device < 64)
+    g_ring_bytes[h->device] -= (long long)h->lz_slabs.size() * h->lz_stride * h->lz_sl;
   h->lz_slabs.clear();
   h->lz_stride = 0;
+}
+static void lz_free(Handle* h) {
+  lz_ring_drop(h);
   for (int slot : {S_LZP, S_LZC})
     if ((int)h->bufs.size() > slot && h->bufs[slot].p) {
       cudaFree(h->bufs[slot].p);
@@ -1073,15 +1083,18 @@ static void lz_free(Handle* h) {
 static int lz_grow(Handle* h, int64_t stride, int sl, int64_t least, int64_t want,
                    size_t budget) {
   if (h->lz_stride != stride || h->lz_sl != sl) {
-    for (void* p : h->lz_slabs) RF_CUDA(cudaFree(p));
-    h->lz_slabs.clear();
+    lz_ring_drop(h);
     h->lz_stride = stride;
     h->lz_sl = sl;
   }
   const size_t bytes = (size_t)stride * sl;
   while ((int64_t)h->lz_slabs.size() * sl < want && h->lz_slabs.size() < (size_t)LZ_SLABS) {
     const bool must = (int64_t)h->lz_slabs.size() * sl < least;
-    if (!must && (h->lz_slabs.size() + 1) * bytes > budget) break;
+    if (!must && ((h->lz_slabs.size() + 1) * bytes > budget ||
+                  (h->device < 64 && h->mem_total &&
+                   g_ring_bytes[h->device] + (long long)bytes >
+                       (long long)(h->mem_total / LZ_RINGS_SHARE))))
+      break;
     void* p = nullptr;
     const cudaError_t e = cudaMalloc(&p, bytes);
     if (e == cudaErrorMemoryAllocation) {
@@ -1091,6 +1104,7 @@ static int lz_grow(Handle* h, int64_t stride, int sl, int64_t least, int64_t wan
     }
     RF_CUDA(e);
     h->lz_slabs.push_back(p);
+    if (h->device < 64) g_ring_bytes[h->device] += (long long)bytes;
   }
   return (int)std::min<int64_t>((int64_t)h->lz_slabs.size() * sl, 1 << 20);
 }
@@ -1940,6 +1954,7 @@ static void filter_lz_batched(std::vector<BatchItem*>& items, Handle* owner, cud
       const int k = ctl[t].iter;
       if (k - k0[t] + steps + 1 > cap[t] && !wrapped[t]) {
         // a batch's rings share a quarter of the device's memory by size
+        h->mem_total = owner->mem_total;
         const size_t budget =
             tight ? 0 : (size_t)(owner->mem_total / 4 * ((double)P[t].a.stride / cells));
         const int got = lz_grow(h, P[t].a.stride, P[t].a.sl, 0, (int64_t)k + steps + 1, budget);
@@ -2598,7 +2613,7 @@ void rafeast_destroy(rafeast_t hh) {
   if (h->stream) cudaStreamSynchronize(h->stream);
   for (auto& b : h->bufs)
     if (b.p) cudaFree(b.p);
-  for (void* p : h->lz_slabs) cudaFree(p);
+  lz_ring_drop(h);
   void* ptrs[] = {h->rowptr, h->colidx, h->val64,   h->val32,   h->perm,  h->iperm,
                   h->Q,      h->AQ,     h->theta_d, h->lrowptr, h->lcolidx, h->trow,
                   h->uoff,   h->ucol,   h->uself,   h->lidx,    h->llidx};
