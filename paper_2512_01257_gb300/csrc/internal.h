@@ -210,11 +210,15 @@ template <typename T> struct LzArgs {
   int64_t stride;  // bytes of a slot: u (n x ld), then t_k and w_j eta_k of every
   int64_t uoff;    // (column, node), double2 pairs, at byte uoff
   T* w;            // L u_k
+  // fixed-point neighbour sums (lanczos.cuh; null: FP64 sums)
+  long long* qu;   // rint(u_k 2^-E), n x ld
+  int* qe;         // [ld] E
+  double rootdeg;  // square root of the greatest degree
   T* dacc;         // quadrature sum, n x ld
   T* p;            // directions: planes (re, im) of node j at p + (2 j) n ld, + n ld
   const double2* z;     // [nc] nodes, the diagonal shift taken off
   const double2* coef;  // [ld * nc] quadrature coefficients
-  double* acc;          // [2 ld] sums of the register-gather product (zeroed)
+  double* acc;          // [3 ld] sums of the register-gather product (zeroed)
   LzCol* col;           // [ld]
   LzShift* sh;          // [ld * nc]
   LzCoef<T>* cf;        // [ld]
@@ -234,7 +238,7 @@ template <typename T>
 void launch_lz_init(const LzArgs<T>& a, const double* q, const double* aq, const double* theta,
                     int ldq, int m, int form, int num_sms, cudaStream_t s);
 template <typename T>
-void launch_lz_dots(const LzArgs<T>& a, int occ, int num_sms, cudaStream_t s);
+void launch_lz_dots(const LzArgs<T>& a, bool fix, int occ, int num_sms, cudaStream_t s);
 template <typename T>
 void launch_lz_update(const LzArgs<T>& a, int num_sms, cudaStream_t s);
 // the steps [k0, k1) into D; last: the solve is over (no direction goes on)
@@ -294,6 +298,7 @@ struct Handle {
   int32_t* lrowptr = nullptr;
   int32_t* lcolidx = nullptr;
   int64_t nnz_off = 0;
+  int max_deg = 0;  // its greatest row (0: unknown, or a row names a column twice)
   // row tiles (ntiles = 0 when the matrix has a row that gathers from more
   // than TILE_UCAP rows): union arrays, and the local indices of the full
   // CSR and of the off-diagonal pattern
@@ -371,7 +376,7 @@ void* scratch(Handle* h, int slot, size_t bytes);  // keep-alive buffer per slot
 void ensure_dyn_smem(const void* fn, size_t bytes);
 enum Slot {
   S_STATE = 0, S_DACC, S_QT, S_TMP1, S_TMP2, S_SCAL, S_GRAM, S_SMALL, S_OMEGA,
-  S_AQ2, S_IO1, S_IO2, S_BATCH, S_TPART, S_SHARD, S_LZ, S_LZP, S_LZC, S_COUNT
+  S_AQ2, S_IO1, S_IO2, S_BATCH, S_TPART, S_SHARD, S_LZ, S_LZP, S_LZC, S_LZQ, S_COUNT
 };
 
 // ---- host math (hostmath.cpp) ------------------------------------------------

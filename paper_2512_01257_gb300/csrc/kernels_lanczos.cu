@@ -35,7 +35,7 @@ __global__ void __launch_bounds__(THREADS) k_lz_init(LzArgs<T> a, const double* 
     x.bad = 0;
     x.kstop = LZ_RUNS;
     a.col[c] = x;
-    a.acc[2 * c] = a.acc[2 * c + 1] = 0.0;
+    for (int t = 0; t < 3; ++t) a.acc[3 * c + t] = 0.0;
     if (c < a.nq) a.qact[c] = 1;
   }
   for (int64_t e = t0; e < (int64_t)a.ld * a.nc; e += st) {
@@ -56,12 +56,13 @@ __global__ void __launch_bounds__(THREADS) k_lz_init(LzArgs<T> a, const double* 
   }
 }
 
-template <typename T, int MAXCPL, int MINB, bool VF>
+template <typename T, int MAXCPL, int MINB, bool VF, bool FX = false>
 __global__ void __launch_bounds__(THREADS, MINB) k_lz_dots(LzArgs<T> a) {
-  lz_dots_body<T, MAXCPL, VF>(a, grid_blk());
+  constexpr int NBX = !FX ? 0 : MAXCPL == 1 && MINB > 3 ? 4 : MAXCPL == 2 && MINB > 2 ? 2 : 0;
+  lz_dots_body<T, MAXCPL, VF, FX, NBX>(a, grid_blk());
 }
 
-template <typename T>
+template <typename T, bool FX>
 __global__ void __launch_bounds__(THREADS) k_lz_update(LzArgs<T> a) {
   // (a CTA with a share of the scalars cannot see `done` set by this step: it
   // waits for every share; the others have no barrier below)
@@ -70,7 +71,7 @@ __global__ void __launch_bounds__(THREADS) k_lz_update(LzArgs<T> a) {
   // contiguous row ranges, CTA 0 at the top
   const int64_t per = (a.n + gridDim.x - 1) / gridDim.x;
   const int64_t r1 = a.n - (int64_t)blockIdx.x * per;
-  if (r1 > 0) lz_update_rows<T>(a, r1 > per ? r1 - per : 0, r1);
+  if (r1 > 0) lz_update_rows<T, FX>(a, r1 > per ? r1 - per : 0, r1);
 }
 
 template <typename T>
@@ -107,10 +108,12 @@ void launch_lz_init(const LzArgs<T>& a, const double* q, const double* aq, const
 }
 
 template <typename T, int MAXCPL, int MINB>
-static void dots_inst(const LzArgs<T>& a, int num_sms, cudaStream_t s) {
-  RF_CHECK(a.cpl <= MAXCPL, RAFEAST_ERR_INVALID_ARG);
+static void dots_inst(const LzArgs<T>& a, bool fix, int num_sms, cudaStream_t s) {
+  RF_CHECK(a.cpl <= MAXCPL && (!fix || a.lcolidx), RAFEAST_ERR_INVALID_ARG);
   auto kern = a.lcolidx ? k_lz_dots<T, MAXCPL, MINB, true> : k_lz_dots<T, MAXCPL, MINB, false>;
-  const size_t smem = lz_dots_smem<T>(a.lanes, MAXCPL, a.ld);
+  if constexpr (sizeof(T) == 8)
+    if (fix) kern = k_lz_dots<T, MAXCPL, MINB, true, true>;
+  const size_t smem = lz_dots_smem<T>(a.lanes, MAXCPL, a.ld, fix ? 3 : 2);
   if (smem > 48 * 1024) ensure_dyn_smem(reinterpret_cast<const void*>(kern), smem);
   const int colblocks = (a.nq + a.lanes * a.cpl - 1) / (a.lanes * a.cpl);
   const int64_t per = (int64_t)WARPS * (32 / a.lanes);
@@ -119,18 +122,19 @@ static void dots_inst(const LzArgs<T>& a, int num_sms, cudaStream_t s) {
   RF_LAUNCH();
 }
 
-// occ: CTAs per SM the instance is compiled for (0: the default of its width)
+// occ: CTAs per SM the instance is compiled for (0: the default of its width);
+// fix: gathers from the fixed-point copy of u_k (a.qu, k > 0)
 template <typename T>
-void launch_lz_dots(const LzArgs<T>& a, int occ, int num_sms, cudaStream_t s) {
+void launch_lz_dots(const LzArgs<T>& a, bool fix, int occ, int num_sms, cudaStream_t s) {
   RF_CHECK(a.lanes > 0 && a.cpl > 0, RAFEAST_ERR_INVALID_ARG);
   if (a.cpl == 1) {
-    if (occ == 3) dots_inst<T, 1, 3>(a, num_sms, s);
-    else dots_inst<T, 1, 4>(a, num_sms, s);
+    if (occ == 3) dots_inst<T, 1, 3>(a, fix, num_sms, s);
+    else dots_inst<T, 1, 4>(a, fix, num_sms, s);
   } else if (a.cpl == 2) {
-    if (occ == 2) dots_inst<T, 2, 2>(a, num_sms, s);
-    else dots_inst<T, 2, 3>(a, num_sms, s);
+    if (occ == 2) dots_inst<T, 2, 2>(a, fix, num_sms, s);
+    else dots_inst<T, 2, 3>(a, fix, num_sms, s);
   } else {
-    dots_inst<T, 4, 2>(a, num_sms, s);
+    dots_inst<T, 4, 2>(a, fix, num_sms, s);
   }
 }
 
@@ -141,7 +145,12 @@ void launch_lz_update(const LzArgs<T>& a, int num_sms, cudaStream_t s) {
   // (at least one CTA per four columns: the scalar shares)
   const int64_t blocks = std::max<int64_t>(
       std::min<int64_t>((a.n + per - 1) / per, (int64_t)num_sms * 6), (a.ld + 3) / 4);
-  k_lz_update<T><<<(int)blocks, THREADS, 0, s>>>(a);
+  if constexpr (sizeof(T) == 8) {
+    if (a.qu) k_lz_update<T, true><<<(int)blocks, THREADS, 0, s>>>(a);
+    else k_lz_update<T, false><<<(int)blocks, THREADS, 0, s>>>(a);
+  } else {
+    k_lz_update<T, false><<<(int)blocks, THREADS, 0, s>>>(a);
+  }
   RF_LAUNCH();
 }
 
@@ -178,7 +187,7 @@ void launch_lz_collapse(const LzArgs<T>& a, int k0, int k1, bool last, int num_s
 #define LZ_INST(T)                                                                             \
   template void launch_lz_init<T>(const LzArgs<T>&, const double*, const double*,              \
                                   const double*, int, int, int, int, cudaStream_t);            \
-  template void launch_lz_dots<T>(const LzArgs<T>&, int, int, cudaStream_t);                   \
+  template void launch_lz_dots<T>(const LzArgs<T>&, bool, int, int, cudaStream_t);             \
   template void launch_lz_update<T>(const LzArgs<T>&, int, cudaStream_t);                      \
   template void launch_lz_collapse<T>(const LzArgs<T>&, int, int, bool, int, cudaStream_t);
 LZ_INST(float)

@@ -89,16 +89,54 @@ __device__ __forceinline__ double2* lz_th(const LzArgs<T>& a, char* slot) {
   return reinterpret_cast<double2*>(slot + a.uoff);
 }
 
-// alpha, g, s of the columns [c0, c1) at step k from their sums (rr, u^T L u at
-// sums[2 (c - c0)], any address space), by the CTA that ends the product
+// Fixed-point neighbour sums (double, LzArgs::qu). FP64 adds issue at 1/64 of
+// the integer rate on this chip, so a neighbour sum of a unit-weight Laplacian
+// is formed in 64-bit integers: the update leaves u_{k+1} a second time as
+// rint(u 2^-E) with one E per column, the product adds those (exactly, modulo
+// 2^64) and returns to FP64 once per row. E is the least exponent for which no
+// sum can leave the range whatever the vector: with N_i the neighbours of i,
+//     |sum_{N_i} u| <= sqrt(max degree) ||u_{k+1}||,
+//     ||u_{k+1}|| <= s (||w - alpha u_k|| + g ||u_{k-1}||),
+// the first norm from the sums u^T u, u^T w, w^T w of the product (a slack of
+// 2^-30 w^T w covers their rounding). The rounding to units of 2^E is an
+// error of w; filter_lz_run takes this path where it cannot exceed the
+// rounding of w = deg u - sum itself. Geometric graph of 16,000 rows (68
+// neighbours, 69 columns): a step of the FP64 filter 218 -> 89 us, product 73 us of it.
 template <typename T>
+__device__ __forceinline__ int lz_fix_exponent(const LzArgs<T>& a, double rr, double ul, double ww,
+                                               double alpha, double g, double s, double rr_prev) {
+  const double t2 = fmax(ww - alpha * (2.0 * ul - alpha * rr), 0.0) + 0x1p-30 * ww;
+  const double x = a.rootdeg * 1.001 * s * (sqrt(t2) + g * sqrt(rr_prev));
+  if (!(x > 0.0) || !isfinite(x)) return 0;
+  return max(-900, min(900, ilogb(x) + 1 - 63));
+}
+// rint(y 2^-E), ties away from zero, in integer arithmetic (FP64 conversions
+// and products would cost more than the sum they prepare)
+__device__ __forceinline__ long long lz_fix(double y, int E) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(y);
+  const int sh = (int)((b >> 52) & 0x7ff) - 1075 - E;  // (a subnormal y is below every unit)
+  unsigned long long m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
+  if (sh >= 0) {
+    m <<= min(sh, 11);  // (11 at most: more means a column of infinities or NaN, which has stopped)
+  } else {
+    const int r = min(-sh, 63);
+    m = (m + (1ull << (r - 1))) >> r;
+  }
+  return (long long)b < 0 ? -(long long)m : (long long)m;
+}
+
+// alpha, g, s of the columns [c0, c1) at step k from their NS sums (rr,
+// u^T L u and, of three, w^T w at sums[NS (c - c0)], any address space), by
+// the CTA that ends the product
+template <typename T, int NS = 2>
 __device__ void lz_column_scalars(const LzArgs<T>& a, int k, int c0, int c1, const double* sums) {
   for (int c = c0 + (int)threadIdx.x; c < c1; c += blockDim.x) {
     LzCol& st = a.col[c];
     LzCoef<T> cf;
     cf.alpha = cf.g = cf.s = cf.pad = (T)0;
+    int E = 0;
     if (st.kstop == LZ_RUNS) {
-      const double rr = sums[2 * (c - c0)], ul = sums[2 * (c - c0) + 1];
+      const double rr = sums[NS * (c - c0)], ul = sums[NS * (c - c0) + 1];
       const double irr = 1.0 / rr, irr_prev = st.irr;
       if (k == 0) st.bnorm2 = rr;
       if (rr > 0.0) {
@@ -110,12 +148,19 @@ __device__ void lz_column_scalars(const LzArgs<T>& a, int k, int c0, int c1, con
           cf.s = cf.alpha != (T)0 ? (T)(1.0 / fabs((double)cf.alpha)) : (T)1;
         }
       }
+      if (sizeof(T) == 8 && a.qe) {
+        // (a step without the third sum: ||L u|| <= 2 (max degree) ||u||)
+        const double ww = NS == 3 ? sums[NS * (c - c0) + 2]
+                                  : 4.0 * a.rootdeg * a.rootdeg * a.rootdeg * a.rootdeg * rr;
+        E = lz_fix_exponent(a, rr, ul, ww, (double)cf.alpha, (double)cf.g, (double)cf.s, st.rr);
+      }
       st.rr = rr;
       st.irr = irr;
       st.bad = !isfinite(rr) || !isfinite(ul) || !isfinite((double)cf.alpha) ||
                !isfinite((double)cf.g) || !isfinite((double)cf.s) || (rr > 0.0 && !(cf.s > (T)0));
     }
     a.cf[c] = cf;
+    if (sizeof(T) == 8 && a.qe) a.qe[c] = E;
   }
 }
 
@@ -278,10 +323,74 @@ __device__ __forceinline__ void lz_scalar_share(const LzArgs<T>& a, int k, int b
 // real columns in the place of a chunk of complex shifts. What bounds it: the
 // latency of the gathers in L1/L2 (float), the FP64 pipe (double).
 // ---------------------------------------------------------------------------
-template <typename T, int MAXCPL, bool VF>
+// the gather core over the fixed-point copy: NB entries in flight, sums modulo
+// 2^64 in any order are the same
+template <int MAXCPL, int NB>
+__device__ __forceinline__ void gather_row_fix(const int32_t* __restrict__ colidx, int k0, int k1,
+                                               int row, int lg, int G, unsigned gmask,
+                                               const long long* __restrict__ X, int64_t ld,
+                                               const int (&coff)[MAXCPL], unsigned mask,
+                                               long long (&acc)[MAXCPL][2]) {
+  for (int kb = k0; kb < k1; kb += G) {
+    const int my_c = kb + lg < k1 ? __ldg(colidx + kb + lg) : row;
+    const int cnt = min(G, k1 - kb);
+    for (int e = 0; e < cnt; e += NB) {
+      int ci[NB];
+#pragma unroll
+      for (int u = 0; u < NB; ++u) ci[u] = __shfl_sync(gmask, my_c, e + u < cnt ? e + u : e, G);
+      longlong2 x[NB][MAXCPL];
+#pragma unroll
+      for (int c = 0; c < MAXCPL; ++c)
+        if (mask & (1u << c)) {
+#pragma unroll
+          for (int u = 0; u < NB; ++u)
+            x[u][c] = __ldg(reinterpret_cast<const longlong2*>(X + (int64_t)ci[u] * ld + coff[c]));
+        }
+      if (e + NB <= cnt) {
+#pragma unroll
+        for (int c = 0; c < MAXCPL; ++c)
+          if (mask & (1u << c)) {
+#pragma unroll
+            for (int u = 0; u < NB; ++u) {
+              acc[c][0] += x[u][c].x;
+              acc[c][1] += x[u][c].y;
+            }
+          }
+      } else {
+#pragma unroll
+        for (int c = 0; c < MAXCPL; ++c)
+          if (mask & (1u << c)) {
+#pragma unroll
+            for (int u = 0; u < NB; ++u)
+              if (e + u < cnt) {
+                acc[c][0] += x[u][c].x;
+                acc[c][1] += x[u][c].y;
+              }
+          }
+      }
+    }
+  }
+}
+// deg u - S 2^E: the two 32-bit halves of S as exact doubles, every factor made
+// from the exponent's bits
+__device__ __forceinline__ double lz_fix_row(long long S, double deg, double u, int E) {
+  // 2^52 + 2^31 + high half, 2^52 + low half
+  const double dh = __hiloint2double(0x43300000, (int)((unsigned long long)S >> 32) ^ 0x80000000);
+  const double dl = __hiloint2double(0x43300000, (int)S);
+  const int x = (E + 1023) << 20;  // (high word of 2^E)
+  // both fma are exact: 2^(E+32) (2^52 + 2^31) = 2^(E+84) (1 + 2^-21)
+  const double h = fma(__hiloint2double((x + (32 << 20)) | 0x80000000, 0), dh,
+                       __hiloint2double(x + (84 << 20), 0x80000000));
+  const double l = fma(__hiloint2double(x | 0x80000000, 0), dl, __hiloint2double(x + (52 << 20), 0));
+  return fma(deg, u, h) + l;
+}
+
+// (NBX: entries in flight, 0: the most the instance's registers hold)
+template <typename T, int MAXCPL, bool VF, bool FX = false, int NBX = 0>
 __device__ __forceinline__ void lz_dots_body(const LzArgs<T>& a, const Blk& blk) {
+  static_assert(!FX || (VF && sizeof(T) == 8), "fixed-point sums: unit weights, double");
   using C = c2<T>;
-  constexpr int NC = sizeof(T) == 4 ? 2 : 1, V = LZV<T>;
+  constexpr int NC = sizeof(T) == 4 ? 2 : 1, V = LZV<T>, NS = FX ? 3 : 2;
   if (__ldcg(&a.ctl->done)) return;
   const RowMap mp = row_map(a.lanes, a.cpl, blk);
   const unsigned gmask = group_mask(mp.G);
@@ -296,11 +405,11 @@ __device__ __forceinline__ void lz_dots_body(const LzArgs<T>& a, const Blk& blk)
     coff[c] = q * V;
     if (c < mp.cpl && q < a.nq && __ldcg(a.qact + q)) mask |= 1u << c;
   }
-  T du[MAXCPL][V], dw[MAXCPL][V];
+  T du[MAXCPL][V], dw[MAXCPL][V], dq[MAXCPL][V];
 #pragma unroll
   for (int c = 0; c < MAXCPL; ++c)
 #pragma unroll
-    for (int v = 0; v < V; ++v) du[c][v] = dw[c][v] = (T)0;
+    for (int v = 0; v < V; ++v) du[c][v] = dw[c][v] = dq[c][v] = (T)0;
   if (__any_sync(0xffffffffu, mask != 0)) {
     const int32_t* __restrict__ rowptr = VF ? a.lrowptr : a.rowptr;
     for (int64_t row = mp.gid; row < a.n; row += mp.gstride) {
@@ -311,8 +420,14 @@ __device__ __forceinline__ void lz_dots_body(const LzArgs<T>& a, const Blk& blk)
 #pragma unroll
         for (int j = 0; j < NC; ++j) acc[c][j] = mk<T>((T)0, (T)0);
       // narrow instances have the registers to keep more entries in flight
-      constexpr int NB = MAXCPL == 1 ? 8 : MAXCPL == 2 ? 4 : 2;
-      if constexpr (VF)
+      constexpr int NB = NBX ? NBX : MAXCPL == 1 ? 8 : MAXCPL == 2 ? 4 : 2;
+      long long fx[MAXCPL][2];
+      if constexpr (FX) {
+#pragma unroll
+        for (int c = 0; c < MAXCPL; ++c) fx[c][0] = fx[c][1] = 0;
+        gather_row_fix<MAXCPL, NB>(a.lcolidx, k0, k1, (int)row, mp.lg, mp.G, gmask, a.qu, a.ld, coff,
+                                   mask, fx);
+      } else if constexpr (VF)
         gather_row_vf<T, NC, MAXCPL, NB>(a.lcolidx, k0, k1, (int)row, mp.lg, mp.G, gmask, U, a.ld,
                                          coff, mask, acc);
       else
@@ -324,10 +439,18 @@ __device__ __forceinline__ void lz_dots_body(const LzArgs<T>& a, const Blk& blk)
         if (mask & (1u << c)) {
           C uv[NC], wv[NC];
           ld_chunk<NC>(U + row * a.ld + coff[c], uv);
+          if constexpr (FX) {
+            // (loaded per row: the registers of the gathers are worth more)
+            int E0, E1;
+            asm volatile("ld.global.v2.s32 {%0, %1}, [%2];" : "=r"(E0), "=r"(E1) : "l"(a.qe + coff[c]));
+            wv[0] = mk<T>(lz_fix_row(fx[c][0], deg, uv[0].x, E0), lz_fix_row(fx[c][1], deg, uv[0].y, E1));
+            dq[c][0] = fma(wv[0].x, wv[0].x, dq[c][0]);
+            dq[c][1] = fma(wv[0].y, wv[0].y, dq[c][1]);
+          }
 #pragma unroll
           for (int j = 0; j < NC; ++j) {
             // values-free: L u = deg u - (sum over neighbours)
-            wv[j] = VF ? mk<T>(fma(deg, uv[j].x, -acc[c][j].x), fma(deg, uv[j].y, -acc[c][j].y))
+            if constexpr (!FX) wv[j] = VF ? mk<T>(fma(deg, uv[j].x, -acc[c][j].x), fma(deg, uv[j].y, -acc[c][j].y))
                        : acc[c][j];
             du[c][2 * j] = fma(uv[j].x, uv[j].x, du[c][2 * j]);
             du[c][2 * j + 1] = fma(uv[j].y, uv[j].y, du[c][2 * j + 1]);
@@ -340,32 +463,34 @@ __device__ __forceinline__ void lz_dots_body(const LzArgs<T>& a, const Blk& blk)
   }
   // groups of a warp by shuffles, warps in shared memory in order, CTAs by
   // global atomics
-  extern __shared__ double sred[];  // [WARPS][G * MAXCPL * V * 2]
-  const int nred = mp.G * MAXCPL * V * 2;
+  extern __shared__ double sred[];  // [WARPS][G * MAXCPL * V * NS]
+  const int nred = mp.G * MAXCPL * V * NS;
 #pragma unroll
   for (int c = 0; c < MAXCPL; ++c)
 #pragma unroll
     for (int v = 0; v < V; ++v) {
-      double x = (double)du[c][v], y = (double)dw[c][v];
+      double x = (double)du[c][v], y = (double)dw[c][v], z = (double)dq[c][v];
       for (int o = mp.G; o < 32; o <<= 1) {
         x += __shfl_xor_sync(0xffffffffu, x, o);
         y += __shfl_xor_sync(0xffffffffu, y, o);
+        if constexpr (FX) z += __shfl_xor_sync(0xffffffffu, z, o);
       }
       if ((threadIdx.x & 31) < mp.G) {
-        double* o = sred + (threadIdx.x >> 5) * nred + ((mp.lg * MAXCPL + c) * V + v) * 2;
+        double* o = sred + (threadIdx.x >> 5) * nred + ((mp.lg * MAXCPL + c) * V + v) * NS;
         o[0] = x;
         o[1] = y;
+        if constexpr (FX) o[2] = z;
       }
     }
   __syncthreads();
   for (int t = threadIdx.x; t < nred; t += blockDim.x) {
-    const int c = (t / (2 * V)) % MAXCPL, lg = t / (2 * V * MAXCPL);
+    const int c = (t / (NS * V)) % MAXCPL, lg = t / (NS * V * MAXCPL);
     const int q = blk.y * mp.G * mp.cpl + lg + c * mp.G;
     if (c < mp.cpl && q < a.nq) {
       double x = 0.0;
 #pragma unroll
       for (int w = 0; w < WARPS; ++w) x += sred[w * nred + t];
-      if (x != 0.0) atomicAdd(&a.acc[2 * (q * V + (t / 2) % V) + (t & 1)], x);
+      if (x != 0.0) atomicAdd(&a.acc[NS * (q * V + (t / NS) % V) + t % NS], x);
     }
     __threadfence();
   }
@@ -375,12 +500,12 @@ __device__ __forceinline__ void lz_dots_body(const LzArgs<T>& a, const Blk& blk)
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  for (int t = threadIdx.x; t < 2 * a.ld; t += blockDim.x) {
+  for (int t = threadIdx.x; t < NS * a.ld; t += blockDim.x) {
     sred[t] = __ldcg(a.acc + t);
     a.acc[t] = 0.0;
   }
   __syncthreads();
-  if (!a.dry) lz_column_scalars<T>(a, k, 0, a.ld, sred);  // (dry: a timing run)
+  if (!a.dry) lz_column_scalars<T, NS>(a, k, 0, a.ld, sred);  // (dry: a timing run)
   if (threadIdx.x == 0) {
     if (!a.dry) lz_advance<T>(a, k);
     a.ctl->ticket = 0;
@@ -388,9 +513,9 @@ __device__ __forceinline__ void lz_dots_body(const LzArgs<T>& a, const Blk& blk)
   }
 }
 template <typename T>
-__host__ __device__ inline size_t lz_dots_smem(int lanes, int maxcpl, int ld) {
-  const size_t red = (size_t)WARPS * lanes * maxcpl * LZV<T> * 2 * sizeof(double);
-  const size_t sc = (size_t)ld * 2 * sizeof(double);
+__host__ __device__ inline size_t lz_dots_smem(int lanes, int maxcpl, int ld, int ns = 2) {
+  const size_t red = (size_t)WARPS * lanes * maxcpl * LZV<T> * ns * sizeof(double);
+  const size_t sc = (size_t)ld * ns * sizeof(double);
   return red > sc ? red : sc;
 }
 
@@ -401,7 +526,8 @@ __host__ __device__ inline size_t lz_dots_smem(int lanes, int maxcpl, int ld) {
 // columns, its coefficients in registers. Bound by HBM: 4 real values per row
 // and column.
 // ---------------------------------------------------------------------------
-template <typename T>
+// FX: u_{k+1} also as rint(u 2^-E) into the fixed-point copy.
+template <typename T, bool FX = false>
 __device__ __forceinline__ void lz_update_rows(const LzArgs<T>& a, int64_t r0, int64_t r1) {
   using Q = typename LzVec<T>::t;
   constexpr int V = LZV<T>, UN = 4;
@@ -409,8 +535,10 @@ __device__ __forceinline__ void lz_update_rows(const LzArgs<T>& a, int64_t r0, i
   const int q = threadIdx.x % nq, rs = threadIdx.x / nq;
   if (rs >= per || !__ldcg(a.qact + q)) return;
   T al[V], g[V], s[V];
+  int E[V];
 #pragma unroll
   for (int v = 0; v < V; ++v) {
+    if constexpr (FX) E[v] = a.qe[q * V + v];
     const LzCoef<T> c = a.cf[q * V + v];
     al[v] = -c.alpha;
     g[v] = -c.g;
@@ -449,6 +577,9 @@ __device__ __forceinline__ void lz_update_rows(const LzArgs<T>& a, int64_t r0, i
           wv[v] = s[v] * y;
         }
         *reinterpret_cast<Q*>(N + rr * a.ld) = lz_put(wv);
+        if constexpr (FX)
+          *reinterpret_cast<longlong2*>(a.qu + rr * a.ld + q * V) =
+              make_longlong2(lz_fix(wv[0], E[0]), lz_fix(wv[1], E[1]));
       }
     }
   }

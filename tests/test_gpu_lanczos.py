@@ -134,3 +134,60 @@ def test_columns_of_extreme_norm(lib):
             assert np.max(np.linalg.norm(y - out[0], axis=0)) <= bound
     finally:
         lib.rafeast_destroy(h)
+
+
+def _dense_graph(kind):
+    rng = np.random.default_rng(5)
+    if kind == "knn":
+        return G.knn3d(601, 10, seed=2, shift=0.2)
+    if kind == "rgg":
+        return G.rgg2d(1500, seed=3, shift=0.2)
+    if kind == "complete":
+        i, j = np.triu_indices(97, 1)
+        return G._from_edges(97, i, j, 0.2, "complete")
+    # one vertex joined to all of a circulant graph of eight neighbours a vertex
+    n, t = 700, np.arange(1, 700)
+    i = np.concatenate([np.zeros(699, int)] + [t] * 4)
+    j = np.concatenate([t] + [1 + (t - 1 + d) % 699 for d in (1, 2, 3, 5)])
+    return G._from_edges(n, i, j, 0.2, "hub")
+
+
+@pytest.mark.parametrize("m0,nc", [(6, 2), (7, 8), (46, 3), (69, 4)])
+@pytest.mark.parametrize("kind", ["knn", "rgg", "complete", "hub"])
+def test_fixed_point_sums_against_dense(lib, kind, m0, nc):
+    """FP64 filter of unit-weight graphs with eight or more neighbours a row
+    (neighbour sums in 64-bit integers) against a dense solve: random columns,
+    one unit vector (the largest entry a column can have), a constant one (no
+    residual after the first step), columns of norm 1e-100 and 1e100, one of
+    entries from 1e-300 to 1.
+
+    Tolerance per unit of ||q||: the stopping rule leaves a residual of 1e-12
+    and the recurrence at most 2^2 eps ||A|| ||x|| per step, so the error of
+    x_j is at most (1e-12 + steps 2^2 eps ||A|| / Im(z_j)) / Im(z_j)."""
+    import torch
+    lap = _dense_graph(kind)
+    A, n, (lo, hi) = lap.scipy().toarray(), lap.n, (0.1, 4.1)
+    q = OF.random_start(n, m0, 1)
+    q[:, 0] = 0.0
+    q[n // 3, 0] = 1.0
+    q[:, 1] = n ** -0.5
+    q[:, 2] *= 1e-100
+    q[:, 3] *= 1e100
+    q[:, 4] = 10.0 ** np.linspace(-300, 0, n)
+    z, w = OQ.nodes(lo, hi, nc, 1.0)
+    exp = sum((wj * np.linalg.solve(zj * np.eye(n) - A, q)).real for zj, wj in zip(z, w))
+    h = lib.rafeast_create(lap.row_ptr, lap.col_idx, lap.values, lap.shift)
+    try:
+        prm = lib.make_params(lo, hi, m0, nc, 1.0, 1e-12, 1e-10, 1, 2000, lib.RAFEAST_FP64,
+                              lib.RAFEAST_FORM_DIRECT)
+        Q = colmajor_dev(q)
+        Qt = torch.zeros_like(Q)
+        info = lib.rafeast_filter(h, prm, Q, None, Qt)
+        assert info.cocg_max_last < 2000
+        got = from_colmajor(Qt)
+    finally:
+        lib.rafeast_destroy(h)
+    norm = np.linalg.norm(q, axis=0)
+    per_step = 4.0 * 2.0 ** -52 * np.abs(A).sum(0).max() * (info.cocg_max_last + 1)
+    tol = np.sum(np.abs(w) * (1e-12 + per_step / z.imag) / z.imag)
+    assert np.max(np.linalg.norm(got - exp, axis=0) / norm) <= tol
