@@ -472,7 +472,7 @@ def run_batched(args):
                                     for t in sorted(range(cnt), key=lambda t: -loop_info[t].t_total_ms)[:4]]}
     peak, peak_kind = _peaks()
     pre = "update" if prof["update_ms"] >= prof["dots_ms"] else "dots"
-    names = {"update": "ms_update_grouped", "dots": "ms_dots_grouped"}
+    names = {"update": "lz_update_grouped", "dots": "lz_dots_grouped"}
     launches_k = max(prof[f"{pre}_launches"], 1.0)
     bytes_per = prof[f"{pre}_bytes"] / launches_k
     ms_per = prof[f"{pre}_ms"] / launches_k
@@ -663,23 +663,21 @@ def _unit_laplacian(lap):
 
 
 def _fp64_dots_roofline(hbm, prof, lap, dev):
-    """The FP64 seed dot kernel is bound by the FP64 pipe, not by HBM: every
-    gathered real entry costs one FP64 add (values-free) or FMA, 1.25 TFLOP/s
-    nominal on this part against 64x that for FP32. Its FP64 lane operations
-    per launch: per active column pair, 4 per gathered entry (two complex
-    columns, real and imaginary parts) and 32 per row (L r from the sum,
-    w = z r - L r, the five dot products). The active pairs come from the
-    library's byte count of the same launches (A once plus, per pair, r read
-    and w written)."""
+    """The FP64 product without fixed-point sums is bound by the FP64 pipe, not
+    by HBM: every gathered entry costs one FP64 add (values-free) or FMA, 1.25
+    TFLOP/s nominal on this part against 64x that for FP32. Its FP64 lane
+    operations per launch: per active column, one per gathered entry and three
+    per row (L u from the sum, the two dot products). The active columns come
+    from the library's byte count of the same launches (A once plus, per
+    column, u read and w written)."""
     import torch
     n = lap.n
     vf, nnz_off = _unit_laplacian(lap)
     abytes = (nnz_off * 4.0 if vf else lap.nnz * 12.0) + 4.0 * (n + 1)
-    pairb = n * 2 * 2.0 * 8.0
     launches = max(prof["dots_launches"], 1.0)
-    act_pairs = (prof["dots_bytes"] - launches * abytes) / (2.0 * pairb)
+    act_cols = (prof["dots_bytes"] - launches * abytes) / (2.0 * 8.0 * n)
     gathered = nnz_off if vf else lap.nnz
-    ops = act_pairs * (4.0 * gathered + 32.0 * n)
+    ops = act_cols * (gathered + 3.0 * n)
     ms = prof["dots_ms"]
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     mhz = 2070.0
@@ -917,10 +915,10 @@ def main():
 
     # roofline of the dominant COCG kernel (live CUDA-event times in the replays)
     peak, peak_kind = _peaks()
-    # multi-shift COCG (default): seed dot kernel k_cocg_dots<.., 2, ..> and
-    # k_ms_update; names of the ncu summaries under profiles/
-    names = {"update": "ms_update_stream",
-             "dots": "ms_dots_tiled" if prof.get("dots_shape", 0) >= 1000000 else "ms_dots"}
+    # real Lanczos form (default): the product k_lz_dots or k_lz_dots_tiled and
+    # k_lz_update; names of the ncu summaries under profiles/
+    names = {"update": "lz_update",
+             "dots": "lz_dots_tiled" if prof.get("dots_shape", 0) >= 1000000 else "lz_dots"}
     pre = "update" if prof["update_ms"] >= prof["dots_ms"] else "dots"
     kern = names[pre]
     launches_k = max(prof[f"{pre}_launches"], 1.0)
@@ -940,12 +938,14 @@ def main():
                                  "ms_per_launch": prof[f"{other}_ms"] / max(prof[f"{other}_launches"], 1)},
                 "share_of_step": (prof["update_ms"] + prof["dots_ms"]) / ms}
 
-    if prec == R.RAFEAST_FP64 and pre == "dots":
+    # (unit-weight Laplacians of eight or more neighbours a row: neighbour sums
+    # in 64-bit integers, which the FP64 pipe does not bind)
+    vf, nnz_off = _unit_laplacian(lap)
+    if prec == R.RAFEAST_FP64 and pre == "dots" and not (vf and nnz_off >= 8 * lap.n):
         roofline = _fp64_dots_roofline(roofline, prof, lap, dev)
-    # the sparse product the metric names: the seed dot kernel, which gathers
-    # w = M r over the CSR pattern (tiled: the gathered rows staged in shared
-    # memory) and forms the step's dot products
-    spmm_kern = "ms_dots_tiled" if prof.get("dots_shape", 0) >= 1000000 else "ms_dots"
+    # the sparse product the metric names: w = L u over the CSR pattern (tiled:
+    # the gathered rows staged in shared memory) with the step's dot products
+    spmm_kern = names["dots"]
     d_launch = max(prof["dots_launches"], 1.0)
     d_bytes = prof["dots_bytes"] / d_launch
     d_ms = prof["dots_ms"] / d_launch
@@ -956,7 +956,7 @@ def main():
                      "algorithmic_bytes_per_launch": d_bytes, "ms_per_launch": d_ms,
                      "launches": int(d_launch), "shape": prof.get("dots_shape"),
                      "algorithmic_bytes": "pattern once (4 B per index, 4 B per row pointer, "
-                                          "values if read) + r read + w written"}
+                                          "values if read) + u read + w written"}
 
     line = {"metric": METRIC, "value": value, "unit": "solves/s", "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_step,
@@ -976,13 +976,11 @@ def main():
             "phases_ms": phases, "roofline": roofline, "roofline_spmm": roofline_spmm,
             "gpu_launches": int(launches), "clocks": ck}
 
-    # COCG working set: seed r, p, w, s and the shifted directions (complex)
-    # plus the quadrature sum
+    # a step's working set: u_{k-1}, u_k, u_{k+1}, w
     sv = 4 if prec == R.RAFEAST_MIXED else 8
-    pairs = (m0 + 1) // 2
-    ws_bytes = n * 2 * pairs * 2 * sv * (4 + (cfg.nc - 1)) + n * 2 * pairs * sv
+    ws_bytes = n * ((m0 + 3) // 4 * 4) * sv * 4
     if ws_bytes < 126e6:
-        line["roofline"]["note"] = (f"COCG working set {ws_bytes / 1e6:.0f} MB fits the 126 MB L2 "
+        line["roofline"]["note"] = (f"a step's working set {ws_bytes / 1e6:.0f} MB fits the 126 MB L2 "
                                     "after the first step: the HBM roofline does not bind")
     if key == "rgg16k":
         # the paper's Table 1 row for this workload: RA-FEAST, N_c = 2,

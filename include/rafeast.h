@@ -100,16 +100,15 @@ extern "C" {
                                      * a lower cap means narrower column       *
                                      * blocks, fewer registers, more warps     */
 #define RAFEAST_OPT_SOLVER 11       /* shifted solves: 0 one COCG per shift,   *
-                                     * 1 multi-shift COCG (one seed recurrence *
-                                     * per column, other shifts from its       *
-                                     * scalars; same iterates in exact         *
-                                     * arithmetic)                              */
-#define RAFEAST_OPT_UPDATE 12       /* multi-shift update kernel: 0 auto    *
-                                     * (streamed), 1 gathered products (M p_k *
-                                     * recomputed from gathered r and p), 2   *
-                                     * streamed (the dot kernel stores M r_k, *
-                                     * M p_k follows by its recurrence; no    *
-                                     * gathers in the update). Batched solves *
+                                     * 1 multi-shift (one recurrence per       *
+                                     * column for every shift; same iterates   *
+                                     * in exact arithmetic)                     */
+#define RAFEAST_OPT_UPDATE 12       /* multi-shift recurrence: 0 real      *
+                                     * Lanczos; complex seed COCG with 1      *
+                                     * gathered products (M p_k recomputed    *
+                                     * from gathered r and p) or 2 a streamed *
+                                     * update (the dot kernel stores M r_k,   *
+                                     * M p_k follows by its recurrence). Batched solves *
                                      * follow the first handle's setting.     */
 #define RAFEAST_OPT_VALUES_FREE 13  /* 0 (default): when the CSR part of A  *
                                      * is a unit-weight graph Laplacian (off- *
@@ -234,8 +233,10 @@ int rafeast_set_option(rafeast_t h, int key, int64_t value);
  * chunks per lane, c the CTAs per SM the chosen kernel instance is compiled
  * for (0: the default instance; dot kernel, update kernel; chosen by the
  * autotuner). Bytes count A once (nnz*(4+s) + 4(n+1), s = 4 or 8) plus each state
- * column the launch reads or writes once: the dot kernel reads r, the update
- * kernel reads r and p, writes r and p, and updates the quadrature sum. With
+ * column the launch reads or writes once: the product reads u_k and writes
+ * L u_k, the update reads both and u_{k-1} and writes u_{k+1} (complex COCG
+ * forms: the dot kernel reads r, the update kernel reads and writes r and p
+ * and updates the quadrature sum). With
  * reset != 0 the counters restart at zero after being copied out. */
 int rafeast_profile(rafeast_t h, int reset, double* out);
 
@@ -400,7 +401,7 @@ int rafeast_solve(rafeast_t h, const rafeast_params* prm, int* m_found,
 /* Solve count independent problems (distinct handles on one device, each
  * with its own params and outputs; arrays of count pointers) as one batch.
  * All problems share precision and nc. Every outer iteration runs the
- * filter of all problems still iterating together: multi-shift COCG (the
+ * filter of all problems still iterating together: multi-shift (the
  * RAFEAST_OPT_SOLVER = 1 path, whatever the handles' options) whose steps
  * are grouped launches, one dot and one update launch per step covering
  * every problem, captured as one CUDA graph on the first handle's stream.
