@@ -251,8 +251,7 @@ __device__ __forceinline__ void lz_nodes(const LzArgs<T>& a, int k, int c, doubl
 }
 
 // the scalar share of CTA b of nb: warp w takes the columns b + nb w,
-// + 8 nb, ...; every CTA with a share (b < nb <= ld) calls it with all its
-// threads. The last of them ends the step.
+// + 8 nb, ...; every CTA with a share (b < nb) calls it with all its threads. The last of them ends the step.
 template <typename T>
 __device__ __forceinline__ void lz_scalar_share(const LzArgs<T>& a, int k, int b, int nb) {
   if (b >= nb) return;
@@ -506,7 +505,8 @@ __device__ __forceinline__ void lz_dots_body(const LzArgs<T>& a, const Blk& blk)
   }
   __syncthreads();
   if (!a.dry) lz_column_scalars<T, NS>(a, k, 0, a.ld, sred);  // (dry: a timing run)
-  if (threadIdx.x == 0) {
+  // (the last thread, which has no column: two latency chains side by side)
+  if (threadIdx.x == blockDim.x - 1) {
     if (!a.dry) lz_advance<T>(a, k);
     a.ctl->ticket = 0;
     __threadfence();
