@@ -253,11 +253,8 @@ void launch_zero(void* p, size_t bytes, cudaStream_t s) {
 constexpr int GRAM_RB = 16;
 
 // SYM: the result is symmetric, so the 16-strided tile blocks below the
-// diagonal (u > v) are skipped; k_gram_sum mirrors them. A: the type the
-// products are formed and summed in within a CTA (double; float for the
-// preconditioning pass of a mixed-precision Cholesky-QR); the CTA partial
-// sums are added in double.
-template <int U, bool SYM, typename A = double>
+// diagonal (u > v) are skipped; k_gram_sum mirrors them.
+template <int U, bool SYM>
 __global__ void __launch_bounds__(256) k_gram_partial(const double* __restrict__ X,
                                                       const double* __restrict__ Y, int64_t n,
                                                       int m, int ld, double* __restrict__ part) {
@@ -265,11 +262,11 @@ __global__ void __launch_bounds__(256) k_gram_partial(const double* __restrict__
   double* Xs = gsm;                 // [GRAM_RB][ld]
   double* Ys = gsm + GRAM_RB * ld;  // [GRAM_RB][ld]
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  A acc[U][U];
+  double acc[U][U];
 #pragma unroll
   for (int u = 0; u < U; ++u)
 #pragma unroll
-    for (int v = 0; v < U; ++v) acc[u][v] = (A)0;
+    for (int v = 0; v < U; ++v) acc[u][v] = 0.0;
   const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
   const int64_t r0 = blockIdx.x * chunk;
   const int64_t r1 = min(n, r0 + chunk);
@@ -283,13 +280,13 @@ __global__ void __launch_bounds__(256) k_gram_partial(const double* __restrict__
     }
     __syncthreads();
     for (int rr = 0; rr < rows; ++rr) {
-      A xa[U], yb[U];
+      double xa[U], yb[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int a = tx + 16 * u;
-        xa[u] = a < m ? (A)Xs[rr * ld + a] : (A)0;
+        xa[u] = a < m ? Xs[rr * ld + a] : 0.0;
         const int b = ty + 16 * u;
-        yb[u] = b < m ? (A)Ys[rr * ld + b] : (A)0;
+        yb[u] = b < m ? Ys[rr * ld + b] : 0.0;
       }
 #pragma unroll
       for (int u = 0; u < U; ++u)
@@ -304,7 +301,75 @@ __global__ void __launch_bounds__(256) k_gram_partial(const double* __restrict__
 #pragma unroll
     for (int v = 0; v < U; ++v) {
       const int a = tx + 16 * u, b = ty + 16 * v;
-      if (a < m && b < m && (!SYM || u <= v)) out[a * m + b] = (double)acc[u][v];
+      if (a < m && b < m && (!SYM || u <= v)) out[a * m + b] = acc[u][v];
+    }
+}
+
+// X^T X of a preconditioning pass, formed and summed in float within a CTA (the
+// CTA partials are added in double): upper tile blocks only. A CTA's rows are one
+// run of memory; the next GRAMF_RB rows' 16-byte loads travel in registers during
+// this stage's products. A value is rounded to float once, on its way to shared
+// memory: conversions issue at the FP64 pipe's rate, and one per use in the
+// product loop cost most of the former kernel: a kNN solve of 200,000 x 80 with 14
+// such passes took 10 ms more, twelve block-model graphs about 50 ms more.
+constexpr int GRAMF_RB = 32;
+template <int U>
+__global__ void __launch_bounds__(256) k_gram_f32(const double* __restrict__ X, int64_t n, int m,
+                                                  int ld, double* __restrict__ part) {
+  extern __shared__ float gsf[];  // [GRAMF_RB][ld]
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  float acc[U][U];
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+#pragma unroll
+    for (int v = 0; v < U; ++v) acc[u][v] = 0.0f;
+  const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
+  const int64_t r0 = blockIdx.x * chunk, r1 = min(n, r0 + chunk);
+  constexpr int NV = GRAMF_RB * 16 * U / 2 / 256;  // (ld <= 16 U; at least 1)
+  const int pairs = GRAMF_RB * ld / 2;
+  double2 nx[NV];
+  auto fetch = [&](int64_t rb) {
+    const int have = (int)min((int64_t)GRAMF_RB, r1 - rb) * ld / 2;
+    const double2* src = reinterpret_cast<const double2*>(X + rb * ld);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const int t = threadIdx.x + 256 * v;
+      nx[v] = t < have ? src[t] : make_double2(0.0, 0.0);
+    }
+  };
+  if (r0 < r1) fetch(r0);
+  for (int64_t rb = r0; rb < r1; rb += GRAMF_RB) {
+    __syncthreads();
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const int t = threadIdx.x + 256 * v;
+      if (t < pairs) reinterpret_cast<float2*>(gsf)[t] = make_float2((float)nx[v].x, (float)nx[v].y);
+    }
+    __syncthreads();
+    if (rb + GRAMF_RB < r1) fetch(rb + GRAMF_RB);
+    const int rows = (int)min((int64_t)GRAMF_RB, r1 - rb);
+#pragma unroll 2
+    for (int rr = 0; rr < rows; ++rr) {
+      float xa[U], yb[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int a = tx + 16 * u, b = ty + 16 * u;
+        xa[u] = a < m ? gsf[rr * ld + a] : 0.0f;
+        yb[u] = b < m ? gsf[rr * ld + b] : 0.0f;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int v = u; v < U; ++v) acc[u][v] = fmaf(xa[u], yb[v], acc[u][v]);
+    }
+  }
+  double* out = part + (int64_t)blockIdx.x * m * m;
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+#pragma unroll
+    for (int v = u; v < U; ++v) {
+      const int a = tx + 16 * u, b = ty + 16 * v;
+      if (a < m && b < m) out[a * m + b] = (double)acc[u][v];
     }
 }
 
@@ -357,17 +422,30 @@ void gram_sum(const double* part, int parts, int m, bool sym, double* G, cudaStr
   RF_LAUNCH();
 }
 
-template <bool SYM, typename A = double>
+template <bool SYM>
 static void gram_partials(const double* X, const double* Y, int64_t n, int m, int ld,
                           double* partial, int parts, size_t smem, cudaStream_t s) {
   switch ((m + 15) / 16) {
 #define RF_GRAM(UU)                                                                      \
   case UU:                                                                               \
-    ensure_dyn_smem(reinterpret_cast<const void*>(k_gram_partial<UU, SYM, A>), smem);   \
-    k_gram_partial<UU, SYM, A><<<parts, 256, smem, s>>>(X, Y, n, m, ld, partial);        \
+    ensure_dyn_smem(reinterpret_cast<const void*>(k_gram_partial<UU, SYM>), smem);      \
+    k_gram_partial<UU, SYM><<<parts, 256, smem, s>>>(X, Y, n, m, ld, partial);           \
     break;
     RF_GRAM(1) RF_GRAM(2) RF_GRAM(3) RF_GRAM(4) RF_GRAM(5) RF_GRAM(6) RF_GRAM(7) RF_GRAM(8)
 #undef RF_GRAM
+    default: throw Err{RAFEAST_ERR_INVALID_ARG};
+  }
+}
+
+static void gram_f32(const double* X, int64_t n, int m, int ld, double* partial, int parts,
+                     cudaStream_t s) {
+  RF_CHECK(ld % 2 == 0 && ld <= (m + 15) / 16 * 16, RAFEAST_ERR_INVALID_ARG);
+  const size_t smem = GRAMF_RB * (size_t)ld * sizeof(float);
+  switch ((m + 15) / 16) {
+#define RF_GRAMF(UU) \
+  case UU: k_gram_f32<UU><<<parts, 256, smem, s>>>(X, n, m, ld, partial); break;
+    RF_GRAMF(1) RF_GRAMF(2) RF_GRAMF(3) RF_GRAMF(4) RF_GRAMF(5) RF_GRAMF(6) RF_GRAMF(7) RF_GRAMF(8)
+#undef RF_GRAMF
     default: throw Err{RAFEAST_ERR_INVALID_ARG};
   }
 }
@@ -379,7 +457,7 @@ void gram(const double* X, const double* Y, int64_t n, int m, int ld, double* G,
   if (f32) {
     // only the symmetric X^T X of a preconditioning pass is formed in float
     if (!sym) throw Err{RAFEAST_ERR_INVALID_ARG};
-    gram_partials<true, float>(X, Y, n, m, ld, partial, parts, smem, s);
+    gram_f32(X, n, m, ld, partial, parts, s);
   } else if (sym) {
     gram_partials<true>(X, Y, n, m, ld, partial, parts, smem, s);
   } else {
