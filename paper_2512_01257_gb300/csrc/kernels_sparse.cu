@@ -461,8 +461,12 @@ __global__ void __launch_bounds__(THREADS) k_shifted_spmm(int64_t n, const int32
   }
 }
 
-template <typename T, int MAXCPL>
-__global__ void __launch_bounds__(THREADS) k_spmm_real(int64_t n, const int32_t* rp,
+// Y = sL L X + sI X. Bound in double by the FP64 pipe (one FMA per entry and
+// value at 2 a clock and SM: 0.45 of the 0.75 ms that 200,000 x 80 with 13.5
+// entries a row take) and by the latency of the gathers. An instance of 8 chunks
+// for every width had the registers for one CTA an SM: 0.77 ms.
+template <typename T, int MAXCPL, int MINB>
+__global__ void __launch_bounds__(THREADS, MINB) k_spmm_real(int64_t n, const int32_t* rp,
                                                        const int32_t* ci, const T* val, int mc,
                                                        int ld, T sL, T sI, const T* X, T* Y,
                                                        int G, int cpl) {
@@ -645,19 +649,32 @@ void launch_shifted_spmm(int64_t n, const int32_t* rp, const int32_t* ci, const 
   }
 }
 
+template <typename T, int MC, int MINB>
+static void spmm_inst(int64_t n, const int32_t* rp, const int32_t* ci, const T* val, int mc, int ld,
+                      T sL, T sI, const T* X, T* Y, int G, int cpl, int blocks, int num_sms,
+                      cudaStream_t s) {
+  auto kern = k_spmm_real<T, MC, MINB>;
+  const int64_t groups = (n + (int64_t)WARPS * (32 / G) - 1) / ((int64_t)WARPS * (32 / G));
+  dim3 grid(grid_x(kern, 0, num_sms, groups), blocks);
+  kern<<<grid, THREADS, 0, s>>>(n, rp, ci, val, mc, ld, sL, sI, X, Y, G, cpl);
+  RF_LAUNCH();
+}
+
 template <typename T>
 void launch_spmm_real(int64_t n, const int32_t* rp, const int32_t* ci, const T* val, int k,
                       int ld, double sL, double sI, const T* X, T* Y, int num_sms,
                       cudaStream_t s) {
-  constexpr int MC = maxcpl_of<T>(1);
   const int mc = (k + 1) / 2;
-  int G, cpl, blocks;
-  choose_shape(mc, 1, sizeof(T) == 8, 0, G, cpl, blocks, 0);
-  auto kern = k_spmm_real<T, MC>;
-  const int64_t groups = (n + (int64_t)WARPS * (32 / G) - 1) / ((int64_t)WARPS * (32 / G));
-  dim3 grid(grid_x(kern, 0, num_sms, groups), blocks);
-  kern<<<grid, THREADS, 0, s>>>(n, rp, ci, val, mc, ld, (T)sL, (T)sI, X, Y, G, cpl);
-  RF_LAUNCH();
+  // eight lanes (128 bytes of a row) and the fewest column blocks of at most 4
+  // chunks a lane. With the layout moves: 200,000 x 80 889 -> 871 us, 2,000 x 24
+  // 30.2 -> 24.4 us.
+  const int G = 8, blocks = (mc + 4 * G - 1) / (4 * G), cpl = (mc + G * blocks - 1) / (G * blocks);
+  if (cpl == 1)
+    spmm_inst<T, 1, 6>(n, rp, ci, val, mc, ld, (T)sL, (T)sI, X, Y, G, cpl, blocks, num_sms, s);
+  else if (cpl == 2)
+    spmm_inst<T, 2, 4>(n, rp, ci, val, mc, ld, (T)sL, (T)sI, X, Y, G, cpl, blocks, num_sms, s);
+  else
+    spmm_inst<T, 4, 2>(n, rp, ci, val, mc, ld, (T)sL, (T)sI, X, Y, G, cpl, blocks, num_sms, s);
 }
 
 // explicit instantiations
