@@ -60,3 +60,45 @@ def test_layout_moves_keep_every_entry(lib, n, k, flag):
         assert np.array_equal(from_colmajor(Y), lap.scipy() @ x)
     finally:
         lib.rafeast_destroy(h)
+
+
+@pytest.mark.parametrize("m", [1, 15, 16, 17, 32, 33, 48, 49, 64, 65, 96, 127, 128])
+def test_block_product_widths(lib, m):
+    """A X over every chunk count and column-block count of the product's
+    instances, with a row longer than one group's index load; a row of d entries
+    and the shift is a chain of d + 2 roundings."""
+    import torch
+    lap = G.knn3d(333, 10, seed=4, shift=0.7)
+    A = lap.scipy().tocsr()
+    x = np.random.default_rng(m).standard_normal((lap.n, m))
+    h = lib.rafeast_create(lap.row_ptr, lap.col_idx, lap.values, lap.shift)
+    try:
+        X = colmajor_dev(x)
+        Y = torch.full_like(X, 7.0)
+        lib.rafeast_spmm(h, m, 1.0, 0.0, X, Y, lib.RAFEAST_FP64)
+        d = np.diff(A.indptr)[:, None] + 2
+        assert np.all(np.abs(from_colmajor(Y) - A @ x) <= 2 * d * 2.0 ** -53 * (abs(A) @ np.abs(x)))
+    finally:
+        lib.rafeast_destroy(h)
+
+
+@pytest.mark.parametrize("n", [140, 601, 9800])
+@pytest.mark.parametrize("m", [1, 15, 16, 17, 33, 64, 65, 127, 128])
+def test_preconditioned_orthonormalisation_widths(lib, m, n):
+    """The warmstart's Cholesky-QR passes (the first of each with a float Gram)
+    at the edges of the Gram's 16-column blocks, with row ranges shorter than a
+    stage, ragged and of several stages: an orthonormal basis whose Ritz values
+    are those of A on it. Backward errors as above, n u ||A||_1, and eight roundings
+    for each of up to 128 columns."""
+    lap = G.knn3d(n, 10, seed=6, shift=0.1)
+    A = lap.scipy()
+    h = lib.rafeast_create(lap.row_ptr, lap.col_idx, lap.values, lap.shift)
+    try:
+        lib.rafeast_warmstart(h, 0.05, 1.0, m, 0, 1, 3)
+        Q = np.zeros((m, n))
+        theta = lib.rafeast_get_subspace(h, Q, m)
+        q, tol = Q.T, (n + 8 * 128) * 2.0 ** -53 * abs(A).sum(0).max()
+        assert np.abs(q.T @ q - np.eye(m)).max() <= tol
+        assert np.abs(q.T @ (A @ q) - np.diag(theta)).max() <= tol
+    finally:
+        lib.rafeast_destroy(h)
