@@ -102,13 +102,19 @@ __device__ __forceinline__ double2* lz_th(const LzArgs<T>& a, char* slot) {
 // error of w; filter_lz_run takes this path where it cannot exceed the
 // rounding of w = deg u - sum itself. Geometric graph of 16,000 rows (68
 // neighbours, 69 columns): a step of the FP64 filter 218 -> 89 us, product 73 us of it.
+// False where the bound leaves the double range (its w^T w does from a norm of
+// about 1e152 on, before the sums of the recurrence do): no unit is safe then.
 template <typename T>
-__device__ __forceinline__ int lz_fix_exponent(const LzArgs<T>& a, double rr, double ul, double ww,
-                                               double alpha, double g, double s, double rr_prev) {
-  const double t2 = fmax(ww - alpha * (2.0 * ul - alpha * rr), 0.0) + 0x1p-30 * ww;
+__device__ __forceinline__ bool lz_fix_exponent(const LzArgs<T>& a, double rr, double ul, double ww,
+                                                double alpha, double g, double s, double rr_prev,
+                                                int& E) {
+  const double au = alpha * ul;  // (at most w^T w)
+  const double t2 = fmax(ww - au - alpha * (ul - alpha * rr), 0.0) + 0x1p-30 * ww;
   const double x = a.rootdeg * 1.001 * s * (sqrt(t2) + g * sqrt(rr_prev));
-  if (!(x > 0.0) || !isfinite(x)) return 0;
-  return max(-900, min(900, ilogb(x) + 1 - 63));
+  E = 0;
+  if (!isfinite(x) || !isfinite(au)) return false;
+  if (x > 0.0) E = max(-900, min(900, ilogb(x) + 1 - 63));
+  return true;
 }
 // rint(y 2^-E), ties away from zero, in integer arithmetic (FP64 conversions
 // and products would cost more than the sum they prepare)
@@ -135,6 +141,7 @@ __device__ void lz_column_scalars(const LzArgs<T>& a, int k, int c0, int c1, con
     LzCoef<T> cf;
     cf.alpha = cf.g = cf.s = cf.pad = (T)0;
     int E = 0;
+    bool unit = true;
     if (st.kstop == LZ_RUNS) {
       const double rr = sums[NS * (c - c0)], ul = sums[NS * (c - c0) + 1];
       const double irr = 1.0 / rr, irr_prev = st.irr;
@@ -152,11 +159,11 @@ __device__ void lz_column_scalars(const LzArgs<T>& a, int k, int c0, int c1, con
         // (a step without the third sum: ||L u|| <= 2 (max degree) ||u||)
         const double ww = NS == 3 ? sums[NS * (c - c0) + 2]
                                   : 4.0 * a.rootdeg * a.rootdeg * a.rootdeg * a.rootdeg * rr;
-        E = lz_fix_exponent(a, rr, ul, ww, (double)cf.alpha, (double)cf.g, (double)cf.s, st.rr);
+        unit = lz_fix_exponent(a, rr, ul, ww, (double)cf.alpha, (double)cf.g, (double)cf.s, st.rr, E);
       }
       st.rr = rr;
       st.irr = irr;
-      st.bad = !isfinite(rr) || !isfinite(ul) || !isfinite((double)cf.alpha) ||
+      st.bad = !unit || !isfinite(rr) || !isfinite(ul) || !isfinite((double)cf.alpha) ||
                !isfinite((double)cf.g) || !isfinite((double)cf.s) || (rr > 0.0 && !(cf.s > (T)0));
     }
     a.cf[c] = cf;

@@ -191,3 +191,38 @@ def test_fixed_point_sums_against_dense(lib, kind, m0, nc):
     per_step = 4.0 * 2.0 ** -52 * np.abs(A).sum(0).max() * (info.cocg_max_last + 1)
     tol = np.sum(np.abs(w) * (1e-12 + per_step / z.imag) / z.imag)
     assert np.max(np.linalg.norm(got - exp, axis=0) / norm) <= tol
+
+
+@pytest.mark.parametrize("kind", ["knn", "rgg"])
+def test_fixed_point_sums_to_the_end_of_the_range(lib, kind):
+    """Columns whose squared norms come near the end of the double range, where
+    the bound on the fixed-point sums leaves it before the sums of the
+    recurrence do: a filter is refused as a breakdown or is right, and it is
+    right up to 2^490 (the greatest degrees are 19 and 70, so ||L||^2 <= 2^15 and
+    w^T w stays in the range up to about 2^504). Tolerance: that of
+    test_fixed_point_sums_against_dense (the powers of two round nothing)."""
+    import torch
+    lap = _dense_graph(kind)
+    A, n, (lo, hi), m0, nc = lap.scipy().toarray(), lap.n, (0.1, 4.1), 6, 4
+    q = OF.random_start(n, m0, 1)
+    z, w = OQ.nodes(lo, hi, nc, 1.0)
+    exp = sum((wj * np.linalg.solve(zj * np.eye(n) - A, q)).real for zj, wj in zip(z, w))
+    h = lib.rafeast_create(lap.row_ptr, lap.col_idx, lap.values, lap.shift)
+    try:
+        prm = lib.make_params(lo, hi, m0, nc, 1.0, 1e-12, 1e-10, 1, 2000, lib.RAFEAST_FP64,
+                              lib.RAFEAST_FORM_DIRECT)
+        for e in [0, 490] + list(range(498, 512)):
+            x = 2.0 ** e
+            Q = colmajor_dev(q * x)
+            Qt = torch.zeros_like(Q)
+            try:
+                info = lib.rafeast_filter(h, prm, Q, None, Qt)
+            except lib.RafeastError as err:
+                assert err.code == lib.RAFEAST_ERR_COCG_BREAKDOWN and e > 490
+                continue
+            err = np.linalg.norm(from_colmajor(Qt) / x - exp, axis=0)
+            per_step = 4.0 * 2.0 ** -52 * np.abs(A).sum(0).max() * (info.cocg_max_last + 1)
+            assert info.cocg_max_last < 2000
+            assert np.max(err) <= np.sum(np.abs(w) * (1e-12 + per_step / z.imag) / z.imag), e
+    finally:
+        lib.rafeast_destroy(h)
