@@ -11,6 +11,12 @@
 
 namespace rafeast {
 
+// tol^2 ||b||^2, against which ||r||^2 is tested; nothing passes where ||b||^2
+// has left the range (an infinite ||r||^2 would: the column is a breakdown)
+__device__ __forceinline__ double stop_threshold(double tol2, double bnorm2) {
+  return isfinite(bnorm2) ? tol2 * bnorm2 : -1.0;
+}
+
 template <typename T>
 __device__ void cocg_scalar_step(const CocgArgs<T>& a, int NC) {
   using C = c2<T>;
@@ -38,7 +44,7 @@ __device__ void cocg_scalar_step(const CocgArgs<T>& a, int NC) {
     if (st.active) {
       if (k == 0) st.bnorm2 = nu;
       if (st.bnorm2 > 0.0) worst = fmax(worst, nu / st.bnorm2);
-      const bool conv = nu <= a.tol2 * st.bnorm2;
+      const bool conv = nu <= stop_threshold(a.tol2, st.bnorm2);
       if (conv || k >= a.max_inner) {
         st.active = 0;
         st.iters = k;
@@ -191,7 +197,7 @@ __device__ void ms_scalar_cols(const CocgArgs<T>& a, int k, int c0, int c1, MsCo
       // the seed system's own stop: its quadrature contribution ends, its
       // recurrence continues while a shifted system of the column needs it.
       // st.iters is -1 while the seed runs, its stop step afterwards.
-      const double thr = a.tol2 * st.bnorm2;
+      const double thr = stop_threshold(a.tol2, st.bnorm2);
       bool any = false;
       bool seed_running = st.iters < 0 || k == 0;
       if (seed_running && (nu <= thr || k >= a.max_inner || !seed_ok)) {
@@ -379,7 +385,7 @@ __device__ void ms_scalar_cols_wide(const CocgArgs<T>& a, int k, int c0, int c1,
       s.bre = bre;
       s.bim = bim;
       s.seed_ok = seed_ok;
-      s.thr = a.tol2 * st.bnorm2;
+      s.thr = stop_threshold(a.tol2, st.bnorm2);
       bool seed_running = st.iters < 0 || k == 0;
       if (seed_running && (nu <= s.thr || k >= a.max_inner || !seed_ok)) {
         if (!(nu <= s.thr)) {

@@ -193,7 +193,7 @@ __device__ __forceinline__ void lz_nodes(const LzArgs<T>& a, int k, int c, doubl
   const LzCol st = a.col[c];
   if (st.kstop != LZ_RUNS) return;
   const double alpha = (double)a.cf[c].alpha, g = (double)a.cf[c].g, s = (double)a.cf[c].s;
-  const double is = 1.0 / s, thr = a.tol2 * st.bnorm2;
+  const double is = 1.0 / s, thr = stop_threshold(a.tol2, st.bnorm2);
   bool run = false, conv = false, brk = false, was = false;
   double worst = 0.0;
   if (j < nc) {

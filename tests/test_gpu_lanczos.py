@@ -226,3 +226,29 @@ def test_fixed_point_sums_to_the_end_of_the_range(lib, kind):
             assert np.max(err) <= np.sum(np.abs(w) * (1e-12 + per_step / z.imag) / z.imag), e
     finally:
         lib.rafeast_destroy(h)
+
+
+@pytest.mark.parametrize("prec,e", [("fp64", 512), ("fp64", 600), ("mixed", 70), ("mixed", 100)])
+@pytest.mark.parametrize("solver,update", [(1, 0), (1, 1), (1, 2), (0, 0)])
+def test_columns_whose_squared_norm_overflows_are_refused(lib, solver, update, prec, e):
+    """||b||^2 outside the range of the working precision: no residual can be
+    compared with it, so no column has converged (an infinite ||r||^2 <= an
+    infinite bound would say so at step 0, with a zero result). (fp64 2^512 times
+    a norm of 2; float entries of about 2^65 and more square to over 2^128.)"""
+    import torch
+    lap = G.grid2d(20, 23, shift=0.3)
+    q0 = 2.0 * OF.random_start(lap.n, 6, 2)
+    h = lib.rafeast_create(lap.row_ptr, lap.col_idx, lap.values, lap.shift)
+    try:
+        lib.rafeast_set_option(h, lib.RAFEAST_OPT_SOLVER, solver)
+        lib.rafeast_set_option(h, lib.RAFEAST_OPT_UPDATE, update)
+        prm = lib.make_params(0.31, 0.6, 6, 4, 1.0, 1e-3, 1e-10, 1, 200,
+                              lib.RAFEAST_FP64 if prec == "fp64" else lib.RAFEAST_MIXED,
+                              lib.RAFEAST_FORM_DIRECT)
+        Q = colmajor_dev(q0 * 2.0 ** e)
+        Qt = torch.zeros_like(Q)
+        with pytest.raises(lib.RafeastError) as ei:
+            lib.rafeast_filter(h, prm, Q, None, Qt)
+        assert ei.value.code == lib.RAFEAST_ERR_COCG_BREAKDOWN
+    finally:
+        lib.rafeast_destroy(h)
