@@ -661,7 +661,9 @@ __device__ __forceinline__ void lz_comp_col(const LzArgs<T>& a, const LzRing& ri
 // D += sum_k c_k u_k over the steps [k0, k1), rows [r0, r1): the pass that ends
 // a solve whose steps all fit the ring. A thread takes RPT rows of one chunk of
 // columns, UB slots' loads in flight together; the coefficients come through
-// L1 (one 16-byte read per RPT rows). Bound by HBM: each u read once.
+// L1 (one 16-byte read per RPT rows). Bound by HBM: each u read once. What a
+// stopped column leaves in later slots (infinite or NaN where its last scale
+// left the range) is not read into D, whatever its neighbours in the chunk do.
 // ---------------------------------------------------------------------------
 template <typename T>
 __device__ __forceinline__ void lz_sum_rows(const LzArgs<T>& a, const LzRing& ring, int cap, int k0,
@@ -671,9 +673,12 @@ __device__ __forceinline__ void lz_sum_rows(const LzArgs<T>& a, const LzRing& ri
   const int nq = a.nq, per = THREADS / nq;
   const int q = threadIdx.x % nq, rs = threadIdx.x / nq;
   if (rs >= per) return;
-  int kq = k0;  // the chunk of columns has coefficients below kq
+  int kq = k0, ks[V];  // the chunk of columns has coefficients below kq, column v below ks[v]
 #pragma unroll
-  for (int v = 0; v < V; ++v) kq = max(kq, min(k1, a.col[q * V + v].kstop));
+  for (int v = 0; v < V; ++v) {
+    ks[v] = a.col[q * V + v].kstop;
+    kq = max(kq, min(k1, ks[v]));
+  }
   for (int64_t r = r0 + rs; r < r1; r += (int64_t)RPT * per) {
     int64_t o[RPT];
     T d[RPT][V];
@@ -703,7 +708,8 @@ __device__ __forceinline__ void lz_sum_rows(const LzArgs<T>& a, const LzRing& ri
             T uv[V];
             lz_get(uq[y][x], uv);
 #pragma unroll
-            for (int v = 0; v < V; ++v) d[x][v] = fma(c[v], uv[v], d[x][v]);
+            for (int v = 0; v < V; ++v)
+              if (k + y < ks[v]) d[x][v] = fma(c[v], uv[v], d[x][v]);
           }
         }
     }
@@ -728,10 +734,11 @@ __device__ __forceinline__ void lz_apply_rows(const LzArgs<T>& a, const LzRing& 
   const int nq = a.nq, nc = a.nc, per = THREADS / nq;
   const int q = threadIdx.x % nq, rs = threadIdx.x / nq;
   if (rs >= per) return;
-  int kq = k0, fl = 0;
+  int kq = k0, fl = 0, ks[V];
 #pragma unroll
   for (int v = 0; v < V; ++v) {
-    kq = max(kq, min(k1, a.col[q * V + v].kstop));
+    ks[v] = a.col[q * V + v].kstop;
+    kq = max(kq, min(k1, ks[v]));
 #pragma unroll
     for (int j = 0; j < JB; ++j)
       if (j0 + j < nc) fl |= a.pflag[(int64_t)(q * V + v) * nc + j0 + j] << (2 * j);
@@ -787,7 +794,12 @@ __device__ __forceinline__ void lz_apply_rows(const LzArgs<T>& a, const LzRing& 
         if (k + y < kq) {
           T uv[RPT][V];
 #pragma unroll
-          for (int x = 0; x < RPT; ++x) lz_get(uq[y][x], uv[x]);
+          for (int x = 0; x < RPT; ++x) {
+            lz_get(uq[y][x], uv[x]);
+#pragma unroll
+            for (int v = 0; v < V; ++v)  // (as in lz_sum_rows)
+              if (k + y >= ks[v]) uv[x][v] = (T)0;
+          }
           if (j0 == 0) {
             T c[V];
             lz_get(__ldg(reinterpret_cast<const Q*>(a.cc + (int64_t)(k + y - k0) * a.ld + q * V)), c);

@@ -252,3 +252,36 @@ def test_columns_whose_squared_norm_overflows_are_refused(lib, solver, update, p
         assert ei.value.code == lib.RAFEAST_ERR_COCG_BREAKDOWN
     finally:
         lib.rafeast_destroy(h)
+
+
+@pytest.mark.parametrize("kind", ["knn", "rgg"])
+def test_a_stopped_column_leaves_its_neighbours_and_result_alone(lib, kind):
+    """A constant column is an eigenvector: it stops at step 1, and near the end
+    of the range the scale of its last vector overflows. Its result, and those of
+    the columns that go on beside it in the same 16 bytes, are those of a dense
+    solve; on both routes of the neighbour sums. Tolerance: that of
+    test_fixed_point_sums_against_dense."""
+    import torch
+    lap = _dense_graph(kind)
+    A, n, (lo, hi), m0, nc = lap.scipy().toarray(), lap.n, (0.1, 4.1), 6, 4
+    q = OF.random_start(n, m0, 1)
+    q[:, 1] = n ** -0.5
+    q[:, 4] = n ** -0.5
+    z, w = OQ.nodes(lo, hi, nc, 1.0)
+    exp = sum((wj * np.linalg.solve(zj * np.eye(n) - A, q)).real for zj, wj in zip(z, w))
+    h = lib.rafeast_create(lap.row_ptr, lap.col_idx, lap.values, lap.shift)
+    try:
+        for values_free in (0, 1):
+            lib.rafeast_set_option(h, lib.RAFEAST_OPT_VALUES_FREE, values_free)
+            prm = lib.make_params(lo, hi, m0, nc, 1.0, 1e-12, 1e-10, 1, 2000, lib.RAFEAST_FP64,
+                                  lib.RAFEAST_FORM_DIRECT)
+            for e in (0, 480, 492, 494, 496, 498):
+                x = 2.0 ** e
+                Q = colmajor_dev(q * x)
+                Qt = torch.zeros_like(Q)
+                info = lib.rafeast_filter(h, prm, Q, None, Qt)
+                err = np.linalg.norm(from_colmajor(Qt) / x - exp, axis=0)
+                per_step = 4.0 * 2.0 ** -52 * np.abs(A).sum(0).max() * (info.cocg_max_last + 1)
+                assert np.max(err) <= np.sum(np.abs(w) * (1e-12 + per_step / z.imag) / z.imag), e
+    finally:
+        lib.rafeast_destroy(h)
