@@ -694,12 +694,16 @@ constexpr size_t JACOBI_SMEM_MAX = 216 * 1024;  // A and V in shared memory up t
 // A (m x m, ld m, symmetric part taken) -> eigenvalues ascending in w, the
 // matching eigenvectors as the columns of Vout (m x m, ld m). A pair (p, q)
 // is rotated while |a_pq| > rot_tol sqrt(|a_pp a_qq|); the sweeps end when
-// the off-diagonal mass is below off_tol of the total, no off-diagonal entry
-// exceeds abs_tol times the root mean square eigenvalue, or a sweep rotated
-// nothing. Vg: global fallback for the eigenvector accumulator (me * me), which
-// is kept transposed (an entry's column-wise neighbours in V, 16 lanes of a
-// warp in one shared-memory bank, made a float round of m = 80 three times as
-// long).
+// the off-diagonal mass is below off_tol of the total or a sweep rotated
+// nothing. An entry below abs_tol times the root mean square eigenvalue is left
+// alone where the pair's eigenvalues are over JACOBI_CLOSE times as far apart: it
+// moves them by less than |a_pq| / JACOBI_CLOSE. In a closer pair it moves them by
+// up to |a_pq| and counts however small it is (three rows with a pair at 2^-30
+// joined by 2^-51: the pair's error with the absolute rule alone was 2^-51).
+// Vg: global fallback for the eigenvector accumulator (me * me), which is kept
+// transposed (an entry's column-wise neighbours in V, 16 lanes of a warp in one
+// shared-memory bank, made a float round of m = 80 three times as long).
+constexpr double JACOBI_CLOSE = 64.0;
 template <typename T>
 __global__ void __launch_bounds__(1024) k_jacobi(const double* __restrict__ Ain, int m, double* __restrict__ w,
                          double* __restrict__ Vout, T* __restrict__ Vg, int max_sweeps,
@@ -712,8 +716,8 @@ __global__ void __launch_bounds__(1024) k_jacobi(const double* __restrict__ Ain,
   T* Vw = (2 * (size_t)me * me * sizeof(T) <= JACOBI_SMEM_MAX) ? A + me * me : Vg;
   __shared__ T cs[64 * 2];  // c, s per pair (me/2 <= 64)
   __shared__ int pq[64 * 2];
-  __shared__ double s_off, s_tot, s_max;
-  __shared__ double s_woff[32], s_wtot[32], s_wmax[32];  // per-warp sums, added in warp order
+  __shared__ double s_off, s_tot;
+  __shared__ double s_woff[32], s_wtot[32];  // per-warp sums, added in warp order
   __shared__ int s_order[128];
   __shared__ int s_rot;
   const T tiny = sizeof(T) == 4 ? (T)1e-37 : (T)1e-300;
@@ -748,41 +752,46 @@ __global__ void __launch_bounds__(1024) k_jacobi(const double* __restrict__ Ain,
       s_rot = 0;
     }
     __syncthreads();
-    double off = 0.0, tot = 0.0, mx = 0.0;
+    double off = 0.0, tot = 0.0;
     for (int t = threadIdx.x; t < me * me; t += blockDim.x) {
       const int i = t / me, j = t % me;
       const double a2 = (double)A[t] * (double)A[t];
       tot += a2;
-      if (i != j) {
-        off += a2;
-        mx = fmax(mx, fabs((double)A[t]));
-      }
+      if (i != j) off += a2;
     }
     off = warp_sum(off);
     tot = warp_sum(tot);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if ((threadIdx.x & 31) == 0) {
       s_woff[threadIdx.x >> 5] = off;
       s_wtot[threadIdx.x >> 5] = tot;
-      s_wmax[threadIdx.x >> 5] = mx;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-      double so = 0.0, st = 0.0, sm = 0.0;
+      double so = 0.0, st = 0.0;
       for (int wi = 0; wi < (int)(blockDim.x >> 5); ++wi) {
         so += s_woff[wi];
         st += s_wtot[wi];
-        sm = fmax(sm, s_wmax[wi]);
       }
       s_off = so;
       s_tot = st;
-      s_max = sm;
     }
     __syncthreads();
     if (!(s_off > off_tol * s_tot) || s_tot == 0.0) break;
     const T small = (T)(abs_tol * sqrt(s_tot / m));
-    if (abs_tol > 0.0 && !(s_max > (double)small)) break;
+    // a_pq is worth a rotation (the square root, an FP64 chain, comes last)
+    auto counts = [&](T apq, T app, T aqq) {
+      const T x = fabs(apq);
+      return x > tiny && (x > small || x * (T)JACOBI_CLOSE > fabs(app - aqq)) &&
+             x > (T)rot_tol * sqrt(fabs(app * aqq));
+    };
+    if (abs_tol > 0.0) {  // no sweep for what is left of the refined matrix, as a rule
+      int any = 0;
+      for (int t = threadIdx.x; t < me * me; t += blockDim.x) {
+        const int i = t / me, j = t % me;
+        if (i < j) any |= counts(A[t], A[i * me + i], A[j * me + j]) ? 1 : 0;
+      }
+      if (!__syncthreads_or(any)) break;
+    }
     for (int round = 0; round < me - 1; ++round) {
       int rotates = 0;
       for (int k = threadIdx.x; k < np; k += blockDim.x) {
@@ -800,8 +809,7 @@ __global__ void __launch_bounds__(1024) k_jacobi(const double* __restrict__ Ain,
         const T apq = A[p * me + q];
         T c = (T)1, s = (T)0;
         const T app = A[p * me + p], aqq = A[q * me + q];
-        if (apq != (T)0 && fabs(apq) > tiny && fabs(apq) > small &&
-            fabs(apq) > (T)rot_tol * sqrt(fabs(app * aqq))) {
+        if (counts(apq, app, aqq)) {
           s_rot = 1;
           rotates = 1;
           const T tau = (aqq - app) / ((T)2 * apq);
@@ -968,8 +976,9 @@ __global__ void __launch_bounds__(128) k_first_order(const double* __restrict__ 
 // steps, square its off-diagonal part for every pair that is not a cluster, by
 // products that run on all SMs; (4) FP64 Jacobi sweeps on what is left, none
 // when every entry is within a few units of rounding (8 eps of the root mean
-// square eigenvalue); (5) V = V1 U1 U2 U3 V_B. On the kNN Rayleigh-Ritz matrix of
-// 80 columns the FP64 part took 2.2 ms as Jacobi sweeps alone.
+// square eigenvalue) and no close pair is coupled; (5) V = V1 U1 U2 U3 V_B. On the
+// kNN Rayleigh-Ritz matrix of 80 columns the FP64 part took 2.2 ms as Jacobi sweeps
+// alone.
 void jacobi_eigh(double* A, int m, double* w, double* V, double* work, cudaStream_t s) {
   if (m > 128) throw Err{RAFEAST_ERR_INVALID_ARG};
   const int me = m + (m & 1);

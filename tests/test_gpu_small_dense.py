@@ -102,3 +102,42 @@ def test_preconditioned_orthonormalisation_widths(lib, m, n):
         assert np.abs(q.T @ (A @ q) - np.diag(theta)).max() <= tol
     finally:
         lib.rafeast_destroy(h)
+
+
+@pytest.mark.parametrize("gap", [0.0, 1.0, 32.0])
+@pytest.mark.parametrize("m", [3, 16, 80])
+def test_close_pair_far_below_the_others_is_resolved(lib, m, gap):
+    """Two eigenvalues near 2^-30 beside ones of order 1, joined by an entry b of
+    a few units of rounding of the large ones, gap b apart: delta + gap b / 2 +-
+    b sqrt(1 + gap^2 / 4). The block is unit vectors, so every product up to the
+    eigensolver is exact, the float stage finds nothing to rotate (b is below its
+    threshold) and one rotation of the pair remains: eight roundings of delta are
+    2^-50 delta, 2^-80, against b of about 2^-50."""
+    n, delta = 200, 2.0 ** -30
+    d = np.full(n, 3.0)
+    d[:m] = 1.0 + np.arange(m)[::-1] / m
+    rms = np.sqrt((d[2:m] ** 2).sum() / m)
+    b = 2.0 ** -52 * (2.0 if m == 3 else 6.0) * 2.0 ** np.floor(np.log2(rms))
+    d[0], d[1] = delta, delta + gap * b
+    rows = [[(i, d[i])] for i in range(n)]
+    rows[0].append((1, b))
+    rows[1].insert(0, (0, b))
+    rp = np.cumsum([0] + [len(r) for r in rows]).astype(np.int32)
+    ci = np.array([c for r in rows for c, _ in r], dtype=np.int32)
+    v = np.array([x for r in rows for _, x in r])
+    q0 = np.zeros((n, m))
+    q0[np.arange(m), np.arange(m)] = 1.0
+    h = lib.rafeast_create(rp, ci, v, 0.0)
+    try:
+        Q = colmajor_dev(q0)
+        theta, _ = lib.rafeast_rayleigh_ritz(h, m, Q)
+        q = from_colmajor(Q)
+    finally:
+        lib.rafeast_destroy(h)
+    root = b * np.sqrt(1.0 + gap * gap / 4.0)
+    exp = delta + gap * b / 2.0 + np.array([-root, root])
+    assert np.max(np.abs(theta[:2] - exp)) <= 2.0 ** -50 * delta
+    # (b, theta - delta) up to scale is an eigenvector: the angle is the same to
+    # 2^-50 delta / b < 2^-28
+    ang = np.arctan2(np.abs(q[1, :2]), np.abs(q[0, :2]))
+    assert np.max(np.abs(ang - np.arctan2(np.abs(exp - delta), b))) <= 2.0 ** -28
