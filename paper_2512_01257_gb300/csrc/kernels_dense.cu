@@ -164,8 +164,14 @@ __global__ void __launch_bounds__(256) k_from_internal(int64_t n, int m,
 // the same one element per thread, for blocks that both levels of cache hold
 // anyway (at most MV_SMALL elements): no shared-memory phase to wait for. 24
 // columns of 2,000 rows: a product with both moves takes 30 us this way, 33 us
-// through shared memory; from about 8 MB on the sectors wasted cost more.
+// through shared memory; from about 8 MB on the sectors wasted cost more. And for
+// blocks of at most MV_NARROW columns at any size, where a CTA's 64 columns would
+// be mostly empty and a row is at most four sectors anyway: float product of
+// 1,000,000 rows with both moves, one column 153 us against 261, 8 columns 242
+// against 322, 14 columns 321 against 379; 200,000 rows 14 columns 119 against
+// 122, 16 columns 124 against 121, 24 columns 165 against 150.
 constexpr int64_t MV_SMALL = 1 << 19;
+constexpr int MV_NARROW = 14;
 __global__ void k_to_internal_small(int64_t n, int m, const double* __restrict__ src,
                                     double* __restrict__ dst, int ld,
                                     const int32_t* __restrict__ iperm) {
@@ -199,7 +205,7 @@ static int blocks_for(int64_t total, int per = 256, int cap = 16384) {
 void launch_to_internal(int64_t n, int m, const double* src, double* dst, int ld,
                         const int32_t* iperm, cudaStream_t s) {
   if (n <= 0 || ld <= 0) return;
-  if (n * (int64_t)ld <= MV_SMALL) {
+  if (n * (int64_t)ld <= MV_SMALL || ld <= MV_NARROW) {
     k_to_internal_small<<<blocks_for(n * (int64_t)ld), 256, 0, s>>>(n, m, src, dst, ld, iperm);
   } else {
     const dim3 grid((unsigned)((n + MV_R - 1) / MV_R), (ld + MV_C - 1) / MV_C);
@@ -211,7 +217,7 @@ void launch_to_internal(int64_t n, int m, const double* src, double* dst, int ld
 void launch_from_internal(int64_t n, int m, const double* src, int ld, double* dst,
                           const int32_t* iperm, const int32_t* cols, cudaStream_t s) {
   if (n <= 0 || m <= 0) return;
-  if (n * (int64_t)m <= MV_SMALL) {
+  if (n * (int64_t)m <= MV_SMALL || m <= MV_NARROW) {
     k_from_internal_small<<<blocks_for(n * (int64_t)m), 256, 0, s>>>(n, m, src, ld, dst, iperm,
                                                                      cols);
   } else {

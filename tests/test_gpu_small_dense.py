@@ -141,3 +141,23 @@ def test_close_pair_far_below_the_others_is_resolved(lib, m, gap):
     # 2^-50 delta / b < 2^-28
     ang = np.arctan2(np.abs(q[1, :2]), np.abs(q[0, :2]))
     assert np.max(np.abs(ang - np.arctan2(np.abs(exp - delta), b))) <= 2.0 ** -28
+
+
+@pytest.mark.parametrize("k", [1, 2, 13, 14, 15, 16])
+@pytest.mark.parametrize("flag", [1, 2])
+def test_narrow_layout_moves_keep_every_entry(lib, k, flag):
+    """As test_layout_moves_keep_every_entry, on both sides of the line between
+    narrow blocks and others where there are more than 2^19 elements (524,309 is
+    odd: ragged last rows)."""
+    import torch
+    n = 524309 if k < 8 else 40009
+    lap = G.cycle(n, 1.0) if hasattr(G, "cycle") else G.grid2d(n, 1, 1.0)
+    x = np.arange(n * k, dtype=np.float64).reshape(n, k) % 1021
+    h = lib.rafeast_create(lap.row_ptr, lap.col_idx, lap.values, lap.shift, flags=flag)
+    try:
+        X = colmajor_dev(x)
+        Y = torch.full_like(X, -1.0)
+        lib.rafeast_spmm(h, k, 1.0, 0.0, X, Y)
+        assert np.array_equal(from_colmajor(Y), lap.scipy() @ x)
+    finally:
+        lib.rafeast_destroy(h)
