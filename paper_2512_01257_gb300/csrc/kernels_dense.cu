@@ -972,6 +972,58 @@ __global__ void __launch_bounds__(128) k_first_order(const double* __restrict__ 
   U[i * m + j] = i == j ? 1.0 : (full[i] || full[j]) ? 0.0 : first_order(B, m, i, j);
 }
 
+// the three rounds of jacobi_eigh's step (3) for m <= REFINE_M in one CTA, one thread
+// per entry and every matrix in shared memory; the sums are those of k_small_gemm.
+// 33 dependent launches of 2 to 3 us are longer than the arithmetic of small
+// matrices: a Rayleigh-Ritz call of 2,000 rows with 1, 4, 8 and 16 columns
+// took 289, 373, 405 and 473 us with them and takes 201, 266, 309 and 414 us.
+constexpr int REFINE_M = 16;
+__global__ void __launch_bounds__(REFINE_M * REFINE_M) k_refine_small(double* __restrict__ Bg,
+                                                                      double* __restrict__ Wg, int m) {
+  using Mat = double[REFINE_M][REFINE_M + 1];
+  __shared__ Mat B, W, U, S;
+  __shared__ int full[REFINE_M];
+  const int i = threadIdx.x / REFINE_M, j = threadIdx.x % REFINE_M;
+  const bool on = i < m && j < m;
+  B[i][j] = on ? Bg[i * m + j] : 0.0;
+  W[i][j] = on ? Wg[i * m + j] : 0.0;
+  __syncthreads();
+  auto first = [&](int r, int c) {  // first_order on the padded rows
+    if (r == c) return 0.0;
+    const double b = 0.5 * (B[r][c] + B[c][r]), gap = B[c][c] - B[r][r];
+    return fabs(b) <= 0.02 * fabs(gap) && gap != 0.0 ? b / gap : 0.0;
+  };
+  // C = alpha op(X) Y + gamma I (every thread has its entry before any is stored)
+  auto gemm = [&](const Mat& X, bool tx, const Mat& Y, Mat& C, double alpha, double gamma) {
+    double acc = 0.0;
+    for (int k = 0; k < m; ++k) acc = fma(tx ? X[k][i] : X[i][k], Y[k][j], acc);
+    __syncthreads();
+    if (on) C[i][j] = alpha * acc + (i == j ? gamma : 0.0);
+    __syncthreads();
+  };
+  for (int it = 0; it < 3; ++it) {
+    if (j == 0 && i < m) {
+      double t = 0.0;
+      for (int c = 0; c < m; ++c) t += fabs(first(i, c));
+      full[i] = !(t <= 0.1);
+    }
+    __syncthreads();
+    if (on) U[i][j] = i == j ? 1.0 : (full[i] || full[j]) ? 0.0 : first(i, j);
+    __syncthreads();
+    for (int ns = 0; ns < 3; ++ns) {
+      gemm(U, true, U, S, -0.5, 1.5);
+      gemm(U, false, S, U, 1.0, 0.0);
+    }
+    gemm(B, false, U, S, 1.0, 0.0);
+    gemm(U, true, S, B, 1.0, 0.0);
+    gemm(W, false, U, W, 1.0, 0.0);
+  }
+  if (on) {
+    Bg[i * m + j] = B[i][j];
+    Wg[i * m + j] = W[i][j];
+  }
+}
+
 // Mixed-precision Jacobi. GB300's FP64 rate is a small fraction of its FP32
 // rate, and a one-CTA FP64 Jacobi sweep of an 80 x 80 matrix takes 0.8 ms of
 // one SM's FP64 issue. So: (1) float Jacobi to the float rounding floor gives
@@ -1003,7 +1055,11 @@ void jacobi_eigh(double* A, int m, double* w, double* V, double* work, cudaStrea
   }
   small_gemm(A, 0, W1, 0, S, m, 1.0, 0.0, s);  // A V
   small_gemm(W1, 1, S, 0, B, m, 1.0, 0.0, s);  // V^T A V
-  for (int it = 0; it < 3; ++it) {
+  if (m <= REFINE_M) {
+    k_refine_small<<<1, REFINE_M * REFINE_M, 0, s>>>(B, W1, m);
+    RF_LAUNCH();
+  }
+  for (int it = 0; it < 3 && m > REFINE_M; ++it) {
     k_first_order_sums<<<m, 128, 0, s>>>(B, m, reinterpret_cast<int*>(S));
     RF_LAUNCH();
     k_first_order<<<m, 128, 0, s>>>(B, m, reinterpret_cast<const int*>(S), VB);

@@ -161,3 +161,10 @@ def test_narrow_layout_moves_keep_every_entry(lib, k, flag):
         assert np.array_equal(from_colmajor(Y), lap.scipy() @ x)
     finally:
         lib.rafeast_destroy(h)
+
+
+@pytest.mark.parametrize("m", [3, 8, 15, 16, 17])
+@pytest.mark.parametrize("kind", ["clusters", "random"])
+def test_rayleigh_ritz_where_the_refinement_changes_kernel(lib, m, kind):
+    """One CTA refines up to 16 columns, products over all SMs more."""
+    test_rayleigh_ritz_is_a_decomposition(lib, m, kind)
