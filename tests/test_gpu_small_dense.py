@@ -168,3 +168,24 @@ def test_narrow_layout_moves_keep_every_entry(lib, k, flag):
 def test_rayleigh_ritz_where_the_refinement_changes_kernel(lib, m, kind):
     """One CTA refines up to 16 columns, products over all SMs more."""
     test_rayleigh_ritz_is_a_decomposition(lib, m, kind)
+
+
+def test_triangular_block_keeps_its_factor(lib):
+    """Columns r e_0 and k e_0 + e_1 with whole r, k: the Gram matrix and both
+    Cholesky columns are exact when the pivot column is divided by r, and r (1/r)
+    is 1 for these r, so R comes back without an error. A product with a rounded
+    1/r misses k by one rounding."""
+    pairs = [(75, 15), (77, 15), (93, 29), (99, 29), (150, 15), (154, 15), (186, 29), (191, 15),
+             (198, 29), (211, 29), (221, 22), (221, 29), (227, 15), (227, 22), (245, 29), (300, 15),
+             (308, 15), (372, 29), (382, 15), (391, 29), (393, 15), (396, 29)]
+    n = 64
+    rp, ci = np.arange(n + 1, dtype=np.int32), np.arange(n, dtype=np.int32)
+    h = lib.rafeast_create(rp, ci, np.ones(n), 0.0)
+    try:
+        for r, k in pairs:
+            x = np.zeros((n, 2))
+            x[0, 0], x[0, 1], x[1, 1] = r, k, 1.0
+            R = lib.rafeast_orthonormalize(h, 2, colmajor_dev(x), want_r=True)
+            assert np.array_equal(R, [[r, k], [0.0, 1.0]]), (r, k, R)
+    finally:
+        lib.rafeast_destroy(h)
