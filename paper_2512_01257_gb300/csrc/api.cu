@@ -1285,11 +1285,17 @@ static void filter_lz_run(Handle* h, const rafeast_params& prm, const double* Qd
   const bool fp64 = sizeof(T) == 8, prof = h->opt_profile != 0;
   cudaStream_t st = h->stream;
   // neighbour sums in fixed point (lanczos.cuh), where FP64 issue bounds the
-  // product and where the rounding to fixed point, at most
-  // sqrt(nnz max_deg / 12) 2.5 2^-62 ||u|| over all rows, stays below the
-  // rounding of w = deg u - sum, 2^-53 sqrt(1 / 12) mean(deg) ||u||:
-  // n max_deg / mean(deg) <= 2^18 / 2.5^2. Rows of fewer than 8 neighbours
-  // gain less than the copy costs.
+  // product and where what they round away stays below what u_{k+1} has lost
+  // already. With N = s (||w - alpha u_k|| + g ||u_{k-1}||) an entry is rounded to
+  // a unit of at most 2^-62 sqrt(max deg) 1.001 N, an error of the neighbour sums
+  // of sqrt(nnz / 12) units (root mean square over all rows). Rounding w - alpha u_k
+  // to FP64 leaves about 2^-53 sqrt(1 / 12) s ||w - alpha u_k|| in u_{k+1}, and the
+  // product multiplies that by the mean degree. w - alpha u_k is the sum of the
+  // orthogonal g u_{k-1} and u_{k+1} / s, so N <= 2 s ||w - alpha u_k||, and the
+  // first is at most the second where n max_deg / mean(deg) <= 2^16; 2^18 / 2.5^2 =
+  // 41,000 leaves a factor of 1.6. (A star and circulant of 600 rows, ratio 36,000,
+  // three steps against 80-bit sums: 1.00 of the error of FP64 sums, geometric mean
+  // over 96 columns.) Rows of fewer than 8 neighbours gain less than the copy costs.
   const bool fixed = fp64 && !tight && h->lcolidx && h->opt_values_free == 0 && h->max_deg > 0 &&
                      h->nnz_off >= 8 * h->n &&
                      (double)h->n * h->n * h->max_deg <= 41000.0 * (double)h->nnz_off;
@@ -1320,7 +1326,7 @@ static void filter_lz_run(Handle* h, const rafeast_params& prm, const double* Qd
         return;
       }
     }
-    launch_lz_dots<T>(ad, fixed, occ, h->num_sms, st);
+    launch_lz_dots<T>(ad, fixed ? LZ_FIX : LZ_PLAIN, occ, h->num_sms, st);
   };
   // autotuner of the product's shape, once per handle, subspace width and
   // precision: the candidates run on u_0 with nothing advancing (a.dry), timed
@@ -1451,12 +1457,12 @@ static void filter_lz_run(Handle* h, const rafeast_params& prm, const double* Qd
   int k0 = 0, cap = (int)h->lz_slabs.size() * a.sl;
   bool wrapped = false;
   const int max_replays = (prm.max_inner + 2) / steps + 2;
-  if (fixed) {  // step 0 by FP64 sums: u_0 has no fixed-point copy
+  if (fixed) {  // step 0 by FP64 sums: u_0 has no fixed-point copy; its w^T w gives u_1's unit
     if (prof) RF_CUDA(cudaEventRecord(evs[0], st));
     LzArgs<T> b = a;
     b.lanes = lanes0;
     b.cpl = cpl0;
-    launch_lz_dots<T>(b, false, 0, h->num_sms, st);
+    launch_lz_dots<T>(b, LZ_SQ, 0, h->num_sms, st);
     if (prof) RF_CUDA(cudaEventRecord(evs[1], st));
     launch_lz_update<T>(a, h->num_sms, st);
     if (prof) {

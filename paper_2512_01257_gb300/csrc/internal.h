@@ -237,8 +237,11 @@ template <typename T> struct LzArgs {
 template <typename T>
 void launch_lz_init(const LzArgs<T>& a, const double* q, const double* aq, const double* theta,
                     int ldq, int m, int form, int num_sms, cudaStream_t s);
+// neighbour sums of the product: plain; plain with w^T w beside the two sums of a
+// column; in fixed point (both double, unit weights)
+enum LzSums { LZ_PLAIN, LZ_SQ, LZ_FIX };
 template <typename T>
-void launch_lz_dots(const LzArgs<T>& a, bool fix, int occ, int num_sms, cudaStream_t s);
+void launch_lz_dots(const LzArgs<T>& a, LzSums sums, int occ, int num_sms, cudaStream_t s);
 template <typename T>
 void launch_lz_update(const LzArgs<T>& a, int num_sms, cudaStream_t s);
 // the steps [k0, k1) into D; last: the solve is over (no direction goes on)

@@ -56,10 +56,10 @@ __global__ void __launch_bounds__(THREADS) k_lz_init(LzArgs<T> a, const double* 
   }
 }
 
-template <typename T, int MAXCPL, int MINB, bool VF, bool FX = false>
+template <typename T, int MAXCPL, int MINB, bool VF, bool FX = false, bool SQ = FX>
 __global__ void __launch_bounds__(THREADS, MINB) k_lz_dots(LzArgs<T> a) {
   constexpr int NBX = !FX ? 0 : MAXCPL == 1 && MINB > 3 ? 4 : MAXCPL == 2 && MINB > 2 ? 2 : 0;
-  lz_dots_body<T, MAXCPL, VF, FX, NBX>(a, grid_blk());
+  lz_dots_body<T, MAXCPL, VF, FX, SQ, NBX>(a, grid_blk());
 }
 
 template <typename T, bool FX>
@@ -111,12 +111,15 @@ void launch_lz_init(const LzArgs<T>& a, const double* q, const double* aq, const
 }
 
 template <typename T, int MAXCPL, int MINB>
-static void dots_inst(const LzArgs<T>& a, bool fix, int num_sms, cudaStream_t s) {
-  RF_CHECK(a.cpl <= MAXCPL && (!fix || a.lcolidx), RAFEAST_ERR_INVALID_ARG);
+static void dots_inst(const LzArgs<T>& a, LzSums sums, int num_sms, cudaStream_t s) {
+  RF_CHECK(a.cpl <= MAXCPL && (sums == LZ_PLAIN || (sizeof(T) == 8 && a.lcolidx && a.qe)),
+           RAFEAST_ERR_INVALID_ARG);
   auto kern = a.lcolidx ? k_lz_dots<T, MAXCPL, MINB, true> : k_lz_dots<T, MAXCPL, MINB, false>;
-  if constexpr (sizeof(T) == 8)
-    if (fix) kern = k_lz_dots<T, MAXCPL, MINB, true, true>;
-  const size_t smem = lz_dots_smem<T>(a.lanes, MAXCPL, a.ld, fix ? 3 : 2);
+  if constexpr (sizeof(T) == 8) {
+    if (sums == LZ_FIX) kern = k_lz_dots<T, MAXCPL, MINB, true, true>;
+    else if (sums == LZ_SQ) kern = k_lz_dots<T, MAXCPL, MINB, true, false, true>;
+  }
+  const size_t smem = lz_dots_smem<T>(a.lanes, MAXCPL, a.ld, sums == LZ_PLAIN ? 2 : 3);
   if (smem > 48 * 1024) ensure_dyn_smem(reinterpret_cast<const void*>(kern), smem);
   const int colblocks = (a.nq + a.lanes * a.cpl - 1) / (a.lanes * a.cpl);
   const int64_t per = (int64_t)WARPS * (32 / a.lanes);
@@ -126,18 +129,19 @@ static void dots_inst(const LzArgs<T>& a, bool fix, int num_sms, cudaStream_t s)
 }
 
 // occ: CTAs per SM the instance is compiled for (0: the default of its width);
-// fix: gathers from the fixed-point copy of u_k (a.qu, k > 0)
+// sums: LZ_FIX gathers from the fixed-point copy of u_k (a.qu, k > 0), LZ_SQ is
+// the step before the first of those
 template <typename T>
-void launch_lz_dots(const LzArgs<T>& a, bool fix, int occ, int num_sms, cudaStream_t s) {
+void launch_lz_dots(const LzArgs<T>& a, LzSums sums, int occ, int num_sms, cudaStream_t s) {
   RF_CHECK(a.lanes > 0 && a.cpl > 0, RAFEAST_ERR_INVALID_ARG);
   if (a.cpl == 1) {
-    if (occ == 3) dots_inst<T, 1, 3>(a, fix, num_sms, s);
-    else dots_inst<T, 1, 4>(a, fix, num_sms, s);
+    if (occ == 3) dots_inst<T, 1, 3>(a, sums, num_sms, s);
+    else dots_inst<T, 1, 4>(a, sums, num_sms, s);
   } else if (a.cpl == 2) {
-    if (occ == 2) dots_inst<T, 2, 2>(a, fix, num_sms, s);
-    else dots_inst<T, 2, 3>(a, fix, num_sms, s);
+    if (occ == 2) dots_inst<T, 2, 2>(a, sums, num_sms, s);
+    else dots_inst<T, 2, 3>(a, sums, num_sms, s);
   } else {
-    dots_inst<T, 4, 2>(a, fix, num_sms, s);
+    dots_inst<T, 4, 2>(a, sums, num_sms, s);
   }
 }
 
@@ -195,7 +199,7 @@ void launch_lz_collapse(const LzArgs<T>& a, int k0, int k1, bool last, int num_s
 #define LZ_INST(T)                                                                             \
   template void launch_lz_init<T>(const LzArgs<T>&, const double*, const double*,              \
                                   const double*, int, int, int, int, cudaStream_t);            \
-  template void launch_lz_dots<T>(const LzArgs<T>&, bool, int, int, cudaStream_t);             \
+  template void launch_lz_dots<T>(const LzArgs<T>&, LzSums, int, int, cudaStream_t);             \
   template void launch_lz_update<T>(const LzArgs<T>&, int, cudaStream_t);                      \
   template void launch_lz_collapse<T>(const LzArgs<T>&, int, int, bool, int, cudaStream_t);
 LZ_INST(float)

@@ -98,9 +98,11 @@ __device__ __forceinline__ double2* lz_th(const LzArgs<T>& a, char* slot) {
 //     |sum_{N_i} u| <= sqrt(max degree) ||u_{k+1}||,
 //     ||u_{k+1}|| <= s (||w - alpha u_k|| + g ||u_{k-1}||),
 // the first norm from the sums u^T u, u^T w, w^T w of the product (a slack of
-// 2^-30 w^T w covers their rounding). The rounding to units of 2^E is an
-// error of w; filter_lz_run takes this path where it cannot exceed the
-// rounding of w = deg u - sum itself. Geometric graph of 16,000 rows (68
+// 2^-30 w^T w covers their rounding; it counts where w is alpha u_k to 2^-15,
+// and is then 2^-15 ||w|| against the 2^-53 ||w|| that w itself is rounded by,
+// far above 2^-62 of the slack). The rounding to units of 2^E is an error of
+// the next w; filter_lz_run takes this path where it stays below the rounding
+// of w - alpha u_k, which u_{k+1} carries anyway. Geometric graph of 16,000 rows (68
 // neighbours, 69 columns): a step of the FP64 filter 218 -> 89 us, product 73 us of it.
 // False where the bound leaves the double range (its w^T w does from a norm of
 // about 1e152 on, before the sums of the recurrence do): no unit is safe then.
@@ -155,19 +157,16 @@ __device__ void lz_column_scalars(const LzArgs<T>& a, int k, int c0, int c1, con
           cf.s = cf.alpha != (T)0 ? (T)(1.0 / fabs((double)cf.alpha)) : (T)1;
         }
       }
-      if (sizeof(T) == 8 && a.qe) {
-        // (a step without the third sum: ||L u|| <= 2 (max degree) ||u||)
-        const double ww = NS == 3 ? sums[NS * (c - c0) + 2]
-                                  : 4.0 * a.rootdeg * a.rootdeg * a.rootdeg * a.rootdeg * rr;
-        unit = lz_fix_exponent(a, rr, ul, ww, (double)cf.alpha, (double)cf.g, (double)cf.s, st.rr, E);
-      }
+      if constexpr (NS == 3)
+        unit = lz_fix_exponent(a, rr, ul, sums[NS * (c - c0) + 2], (double)cf.alpha, (double)cf.g,
+                               (double)cf.s, st.rr, E);
       st.rr = rr;
       st.irr = irr;
       st.bad = !unit || !isfinite(rr) || !isfinite(ul) || !isfinite((double)cf.alpha) ||
                !isfinite((double)cf.g) || !isfinite((double)cf.s) || (rr > 0.0 && !(cf.s > (T)0));
     }
     a.cf[c] = cf;
-    if (sizeof(T) == 8 && a.qe) a.qe[c] = E;
+    if constexpr (NS == 3) a.qe[c] = E;
   }
 }
 
@@ -391,12 +390,13 @@ __device__ __forceinline__ double lz_fix_row(long long S, double deg, double u, 
   return fma(deg, u, h) + l;
 }
 
-// (NBX: entries in flight, 0: the most the instance's registers hold)
-template <typename T, int MAXCPL, bool VF, bool FX = false, int NBX = 0>
+// (SQ: w^T w as a third sum, from which the fixed-point unit of u_{k+1} is made;
+// NBX: entries in flight, 0: the most the instance's registers hold)
+template <typename T, int MAXCPL, bool VF, bool FX = false, bool SQ = FX, int NBX = 0>
 __device__ __forceinline__ void lz_dots_body(const LzArgs<T>& a, const Blk& blk) {
   static_assert(!FX || (VF && sizeof(T) == 8), "fixed-point sums: unit weights, double");
   using C = c2<T>;
-  constexpr int NC = sizeof(T) == 4 ? 2 : 1, V = LZV<T>, NS = FX ? 3 : 2;
+  constexpr int NC = sizeof(T) == 4 ? 2 : 1, V = LZV<T>, NS = SQ ? 3 : 2;
   if (__ldcg(&a.ctl->done)) return;
   const RowMap mp = row_map(a.lanes, a.cpl, blk);
   const unsigned gmask = group_mask(mp.G);
@@ -450,8 +450,6 @@ __device__ __forceinline__ void lz_dots_body(const LzArgs<T>& a, const Blk& blk)
             int E0, E1;
             asm volatile("ld.global.v2.s32 {%0, %1}, [%2];" : "=r"(E0), "=r"(E1) : "l"(a.qe + coff[c]));
             wv[0] = mk<T>(lz_fix_row(fx[c][0], deg, uv[0].x, E0), lz_fix_row(fx[c][1], deg, uv[0].y, E1));
-            dq[c][0] = fma(wv[0].x, wv[0].x, dq[c][0]);
-            dq[c][1] = fma(wv[0].y, wv[0].y, dq[c][1]);
           }
 #pragma unroll
           for (int j = 0; j < NC; ++j) {
@@ -462,6 +460,10 @@ __device__ __forceinline__ void lz_dots_body(const LzArgs<T>& a, const Blk& blk)
             du[c][2 * j + 1] = fma(uv[j].y, uv[j].y, du[c][2 * j + 1]);
             dw[c][2 * j] = fma(uv[j].x, wv[j].x, dw[c][2 * j]);
             dw[c][2 * j + 1] = fma(uv[j].y, wv[j].y, dw[c][2 * j + 1]);
+            if constexpr (SQ) {
+              dq[c][2 * j] = fma(wv[j].x, wv[j].x, dq[c][2 * j]);
+              dq[c][2 * j + 1] = fma(wv[j].y, wv[j].y, dq[c][2 * j + 1]);
+            }
           }
           st_chunk<NC>(a.w + row * a.ld + coff[c], wv);
         }
@@ -479,13 +481,13 @@ __device__ __forceinline__ void lz_dots_body(const LzArgs<T>& a, const Blk& blk)
       for (int o = mp.G; o < 32; o <<= 1) {
         x += __shfl_xor_sync(0xffffffffu, x, o);
         y += __shfl_xor_sync(0xffffffffu, y, o);
-        if constexpr (FX) z += __shfl_xor_sync(0xffffffffu, z, o);
+        if constexpr (SQ) z += __shfl_xor_sync(0xffffffffu, z, o);
       }
       if ((threadIdx.x & 31) < mp.G) {
         double* o = sred + (threadIdx.x >> 5) * nred + ((mp.lg * MAXCPL + c) * V + v) * NS;
         o[0] = x;
         o[1] = y;
-        if constexpr (FX) o[2] = z;
+        if constexpr (SQ) o[2] = z;
       }
     }
   __syncthreads();
