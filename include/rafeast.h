@@ -211,6 +211,25 @@ int rafeast_create(rafeast_t* out, int64_t n, int64_t nnz,
                    const double* values, double diag_shift,
                    int inputs_on_device, void* stream, uint32_t flags);
 
+/* Memory. A handle keeps its workspaces and, for the default multi-shift
+ * recurrence, a ring of Lanczos vectors (RAFEAST_OPT_UPDATE 0) for its next call.
+ * A ring takes the chunk of RAFEAST_OPT_CHUNK + 2 vectors that a replay needs;
+ * beyond that it grows with the steps of a filter to at most a sixteenth of the
+ * device's memory, all rings on a device together to a quarter. When an allocation of the library fails, or
+ * a ring may not grow otherwise, rings of handles that are not in a filter are
+ * taken back first, the longest unused before the others; a filter that still
+ * runs out of memory is run once more with the smallest ring. */
+
+/* Memory. A handle keeps its workspaces and, for the default multi-shift
+ * recurrence (RAFEAST_OPT_UPDATE 0), a ring of Lanczos vectors for its next
+ * filter. A ring holds the RAFEAST_OPT_CHUNK + 2 vectors that a replay needs;
+ * beyond those it grows with the steps of a filter to at most a sixteenth of the
+ * device's memory, all rings on a device together to a quarter, and only while a
+ * sixteenth of the device stays free. When an allocation of the library fails, or
+ * a ring may not grow otherwise, rings of handles that are in no filter are taken
+ * back, the longest unused first; a filter that still runs out of memory is run
+ * once more with the smallest ring. */
+
 /* Release the handle and all its device memory. NULL is a no-op. */
 void rafeast_destroy(rafeast_t h);
 

@@ -74,6 +74,71 @@ void ensure_dyn_smem(const void* fn, size_t bytes) {
   set.push_back(std::make_pair(std::make_pair(dev, fn), bytes));
 }
 
+// ---- rings of Lanczos vectors (lanczos.cuh) -----------------------------------
+// A handle keeps the slabs of its ring for its next filter. This list has every
+// handle that holds some, the longest unused first, so that memory which is asked
+// for and not to be had comes from rings that no filter is using, whichever
+// handle asks.
+static std::mutex g_ring_mu;
+static std::vector<Handle*> g_rings;
+static size_t ring_bytes(int device) {  // (the mutex is held)
+  size_t b = 0;
+  for (const Handle* r : g_rings)
+    if (r->device == device) b += r->lz_slabs.size() * r->lz_slab_bytes;
+  return b;
+}
+static void ring_drop_locked(Handle* h) {
+  if (h->lz_slabs.empty()) return;
+  cudaEventSynchronize(h->lz_done);
+  for (void* p : h->lz_slabs) cudaFree(p);
+  h->lz_slabs.clear();
+  h->lz_slab_bytes = 0;
+  g_rings.erase(std::find(g_rings.begin(), g_rings.end(), h));
+}
+static void lz_ring_drop(Handle* h) {
+  std::lock_guard<std::mutex> lock(g_ring_mu);
+  ring_drop_locked(h);
+}
+// the longest unused ring of the device goes back to it; false: there is none
+static bool ring_reclaim_locked(int device) {
+  for (Handle* r : g_rings)
+    if (r->device == device && !r->lz_busy) {
+      ring_drop_locked(r);
+      return true;
+    }
+  return false;
+}
+// a handle's ring is in use while one of these lives; its end is behind the
+// filter's launches on the handle's stream
+struct RingUse {
+  Handle* h;
+  explicit RingUse(Handle* hh) : h(hh) {
+    std::lock_guard<std::mutex> lock(g_ring_mu);
+    h->lz_busy = true;
+    auto it = std::find(g_rings.begin(), g_rings.end(), h);
+    if (it != g_rings.end()) std::rotate(it, it + 1, g_rings.end());
+  }
+  ~RingUse() {
+    std::lock_guard<std::mutex> lock(g_ring_mu);
+    cudaEventRecord(h->lz_done, h->stream);
+    h->lz_busy = false;
+  }
+  RingUse(const RingUse&) = delete;
+  RingUse& operator=(const RingUse&) = delete;
+};
+
+// cudaMalloc on the current device that takes idle rings back before it fails
+template <typename T>
+static cudaError_t dev_malloc(int device, T** p, size_t bytes) {
+  for (;;) {
+    const cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    std::lock_guard<std::mutex> lock(g_ring_mu);
+    if (!ring_reclaim_locked(device)) return e;
+    cudaGetLastError();
+  }
+}
+
 void* scratch(Handle* h, int slot, size_t bytes) {
   if ((int)h->bufs.size() <= slot) h->bufs.resize(slot + 1);
   DevBuf& b = h->bufs[slot];
@@ -82,7 +147,7 @@ void* scratch(Handle* h, int slot, size_t bytes) {
     if (b.p) RF_CUDA(cudaFree(b.p));
     b.p = nullptr;
     b.bytes = 0;
-    RF_CUDA(cudaMalloc(&b.p, bytes));
+    RF_CUDA(dev_malloc(h->device, &b.p, bytes));
     b.bytes = bytes;
   }
   return b.p;
@@ -1051,25 +1116,17 @@ struct LzProblem {
   LzArgs<T> a;
   const double* fin = nullptr;  // device [m0]: per-column constant of the correction form
   int m0 = 0;
+  int cap = 0;  // slots of the ring
 };
 
 // ---- the ring of Lanczos vectors (Handle::lz_slabs) ---------------------------
-// Slots are allocated as a solve needs them, up to a share of the device's
-// memory (LZ_RING_SHARE); a solve with more steps than slots folds full rings
-// into its directions. A slab is about a gigabyte or the whole of 32 slots.
-// All handles' rings on a device together grow to a quarter of its memory at
-// most (beyond the slots a replay cannot do without), so that many handles
-// kept side by side leave room for the program's own tensors.
-constexpr size_t LZ_RING_SHARE = 16;  // a sixteenth of the device's memory
-constexpr size_t LZ_RINGS_SHARE = 4;  // all rings
-static std::atomic<long long> g_ring_bytes[64];  // by device (a larger index: not bounded)
-static void lz_ring_drop(Handle* h) {
-  for (void* p : h->lz_slabs) cudaFree(p);
-  if (h->device < 64)
-    g_ring_bytes[h->device] -= (long long)h->lz_slabs.size() * h->lz_stride * h->lz_sl;
-  h->lz_slabs.clear();
-  h->lz_stride = 0;
-}
+// Slots are allocated as a solve needs them. Beyond the slots a replay cannot do
+// without, a ring grows to a share of the device's memory (LZ_RING_SHARE), all
+// rings on the device together to a quarter of it; a solve with more steps than
+// slots folds full rings into its directions.
+constexpr size_t LZ_RING_SHARE = 16;   // one ring: a sixteenth of the device's memory
+constexpr size_t LZ_RINGS_SHARE = 4;   // all rings
+constexpr int LZ_MAX_SL = 4096;        // slots of a slab made for larger ones
 static void lz_free(Handle* h) {
   lz_ring_drop(h);
   for (int slot : {S_LZP, S_LZC, S_LZQ})
@@ -1078,44 +1135,73 @@ static void lz_free(Handle* h) {
       h->bufs[slot] = DevBuf();
     }
 }
-// slots of `stride` bytes: `least` of them, or it throws, and `want` if they
-// can be had within `budget` bytes; returns the slots there are
-static int lz_grow(Handle* h, int64_t stride, int sl, int64_t least, int64_t want,
-                   size_t budget) {
-  if (h->lz_stride != stride || h->lz_sl != sl) {
-    lz_ring_drop(h);
-    h->lz_stride = stride;
-    h->lz_sl = sl;
-  }
-  const size_t bytes = (size_t)stride * sl;
+// what a filter may take of the ring
+struct LzRoom {
+  bool tight = false;  // the smallest ring
+  int steps = 2;       // steps per graph replay (even)
+  int limit = 0;       // most slots (0: no limit of its own)
+  double share = 1.0 / LZ_RING_SHARE;  // of the device's memory, for slots beyond the least
+  int per_slab() const { return limit ? std::min(limit, LZ_SL) : LZ_SL; }
+  int least() const { return steps + 2; }  // a replay's slots and u_{k0-1}
+};
+static LzRoom lz_room(const Handle* h, bool tight) {
+  LzRoom r;
+  r.tight = tight;
+  r.limit = tight ? 4 : 0;
+  r.steps = std::min(62, std::max(2, h->opt_chunk + (h->opt_chunk & 1)));
+  if (r.limit) r.steps = std::min(r.steps, std::max(2, (r.limit - 2) & ~1));
+  return r;
+}
+static int lz_slab_slots(const Handle* h, int64_t stride) {
+  return (int)std::min<int64_t>(LZ_MAX_SL, (int64_t)h->lz_slab_bytes / stride);
+}
+// slots of `stride` bytes: the least a replay needs, or it throws, and `want` of
+// them as far as there is room; returns the slots there are. A slab holds 32
+// slots of up to 32 MB, is a gigabyte while that is 8 slots, and 8 slots above.
+static int lz_grow(Handle* h, int64_t stride, const LzRoom& room, int64_t want) {
+  const int64_t per = room.per_slab(), gb = (int64_t)1 << 30;
+  int64_t slab = stride * per;
+  if (slab > gb) slab = std::max(gb, stride * std::min<int64_t>(per, 8));
+  std::lock_guard<std::mutex> lock(g_ring_mu);
+  if ((int64_t)h->lz_slab_bytes != slab) ring_drop_locked(h);
+  if (h->lz_slabs.empty()) h->lz_slab_bytes = (size_t)slab;
+  const size_t bytes = h->lz_slab_bytes;
+  const int64_t sl = lz_slab_slots(h, stride), least = room.least();
+  if (room.limit) want = std::min<int64_t>(want, room.limit);
+  want = std::max(want, least);
   while ((int64_t)h->lz_slabs.size() * sl < want && h->lz_slabs.size() < (size_t)LZ_SLABS) {
-    const bool must = (int64_t)h->lz_slabs.size() * sl < least;
-    if (!must && ((h->lz_slabs.size() + 1) * bytes > budget ||
-                  (h->device < 64 && h->mem_total &&
-                   g_ring_bytes[h->device] + (long long)bytes >
-                       (long long)(h->mem_total / LZ_RINGS_SHARE))))
-      break;
+    if ((int64_t)h->lz_slabs.size() * sl >= least) {
+      size_t mem_free = 0, total = 0;
+      RF_CUDA(cudaMemGetInfo(&mem_free, &total));
+      if ((double)(h->lz_slabs.size() + 1) * bytes > room.share * total) break;
+      if (ring_bytes(h->device) + bytes > total / LZ_RINGS_SHARE) {
+        if (!ring_reclaim_locked(h->device)) break;
+        continue;
+      }
+    }
     void* p = nullptr;
     const cudaError_t e = cudaMalloc(&p, bytes);
     if (e == cudaErrorMemoryAllocation) {
       cudaGetLastError();
-      if (!must) break;
+      if (ring_reclaim_locked(h->device)) continue;
+      if ((int64_t)h->lz_slabs.size() * sl >= least) break;
       throw Err{RAFEAST_ERR_OUT_OF_MEMORY};
     }
     RF_CUDA(e);
+    if (h->lz_slabs.empty()) g_rings.push_back(h);
     h->lz_slabs.push_back(p);
-    if (h->device < 64) g_ring_bytes[h->device] += (long long)bytes;
   }
-  return (int)std::min<int64_t>((int64_t)h->lz_slabs.size() * sl, 1 << 20);
+  const int64_t cap = (int64_t)h->lz_slabs.size() * sl;
+  return (int)(room.limit ? std::min<int64_t>(cap, std::max<int64_t>(room.limit, least)) : cap);
 }
 
 // the slab table and the slot count to the device (no step in flight)
 template <typename T>
-static void lz_ring_upload(Handle* h, const LzArgs<T>& a, cudaStream_t st) {
+static void lz_ring_upload(Handle* h, const LzArgs<T>& a, int cap, cudaStream_t st) {
   LzDyn d;
   memset(&d, 0, sizeof(d));
   for (size_t t = 0; t < h->lz_slabs.size(); ++t) d.slab[t] = (char*)h->lz_slabs[t];
-  d.cap = (int)h->lz_slabs.size() * a.sl;
+  d.cap = cap;
   RF_CUDA(cudaMemcpyAsync(a.dyn, &d, offsetof(LzDyn, k), cudaMemcpyHostToDevice, st));
 }
 
@@ -1133,19 +1219,13 @@ static void lz_collapse(Handle* h, LzArgs<T> a, int k0, int k1, bool last, cudaS
   h->launches += dirs ? 1 + (a.nc + 3) / 4 : 2;
 }
 
-// steps per graph replay (even)
-static int lz_replay_steps(const Handle* h, bool tight) {
-  if (tight) return 2;
-  return std::min(62, std::max(2, h->opt_chunk + (h->opt_chunk & 1)));
-}
-
 // quadrature, coefficient upload and state init of one problem on stream st
 // (one launch). ctl_dev replaces the handle's own control block (batches).
 template <typename T>
 static LzProblem<T> lz_setup(Handle* h, const rafeast_params& prm, const double* Qd,
                              const double* AQd, const double* theta_d,
                              const std::vector<double>& theta, int m0, int ldq, CocgCtl* ctl_dev,
-                             bool profile, bool tight, bool fixed, cudaStream_t st) {
+                             bool profile, const LzRoom& room, bool fixed, cudaStream_t st) {
   const bool fp64 = sizeof(T) == 8;
   std::vector<double> zr, zi, wr, wi;
   quadrature_nodes(prm.lmin, prm.lmax, prm.nc, prm.ellipse_ratio, zr, zi, wr, wi);
@@ -1189,16 +1269,15 @@ static LzProblem<T> lz_setup(Handle* h, const rafeast_params& prm, const double*
   const int64_t block = h->n * (int64_t)ld * sizeof(T);
   a.uoff = (block + 255) & ~(int64_t)255;
   a.stride = (a.uoff + (int64_t)sizeof(double2) * 2 * ld * nc + 255) & ~(int64_t)255;
-  // 32 slots a slab, fewer when that is over a gigabyte; 4 when memory is short
-  a.sl = tight ? 4 : (int)std::max<int64_t>(8, std::min<int64_t>(LZ_SL, ((int64_t)1 << 30) / a.stride));
   int blocks = 1;
   choose_shape(nq, 2, fp64, h->opt_lanes, a.lanes, a.cpl, blocks,
                h->opt_cpl > 0 ? std::min(h->opt_cpl, 4) : 2);
   a.w = (T*)scratch(h, S_STATE, block);
   a.dacc = (T*)scratch(h, S_DACC, block);
-  const int least = lz_replay_steps(h, tight) + 2;  // a replay's slots and u_{k0-1}
-  lz_grow(h, a.stride, a.sl, least, least, 0);
-  if (tight) scratch(h, S_LZP, (size_t)2 * nc * block);
+  LzProblem<T> P;
+  P.cap = lz_grow(h, a.stride, room, 0);
+  a.sl = lz_slab_slots(h, a.stride);
+  if (room.tight) scratch(h, S_LZP, (size_t)2 * nc * block);
   size_t off = 0;
   auto carve = [&](size_t bytes) {
     off = (off + 255) & ~(size_t)255;
@@ -1242,10 +1321,9 @@ static LzProblem<T> lz_setup(Handle* h, const rafeast_params& prm, const double*
   a.rhist = profile ? (double*)(sc + o_rhist) : nullptr;
   a.tol2 = prm.solve_tol * prm.solve_tol;
   a.max_inner = prm.max_inner;
-  lz_ring_upload(h, a, st);
+  lz_ring_upload(h, a, P.cap, st);
   launch_lz_init<T>(a, Qd, AQd, theta_d, ldq, m0, prm.solve_form, h->num_sms, st);
   h->launches += 1;
-  LzProblem<T> P;
   P.a = a;
   P.fin = (const double*)(sc + o_up) + 2 * (n_z + n_coef);
   P.m0 = m0;
@@ -1299,8 +1377,10 @@ static void filter_lz_run(Handle* h, const rafeast_params& prm, const double* Qd
   const bool fixed = fp64 && !tight && h->lcolidx && h->opt_values_free == 0 && h->max_deg > 0 &&
                      h->nnz_off >= 8 * h->n &&
                      (double)h->n * h->n * h->max_deg <= 41000.0 * (double)h->nnz_off;
+  const LzRoom room = lz_room(h, tight);
+  RingUse use(h);
   LzProblem<T> P =
-      lz_setup<T>(h, prm, Qd, AQd, theta_d, theta, m0, ldq, nullptr, prof, tight, fixed, st);
+      lz_setup<T>(h, prm, Qd, AQd, theta_d, theta, m0, ldq, nullptr, prof, room, fixed, st);
   LzArgs<T>& a = P.a;
   const bool vf = a.lcolidx != nullptr;
   const bool can_tile = !fp64 && h->ntiles > 0 && h->opt_tiled != 1 &&
@@ -1412,7 +1492,7 @@ static void filter_lz_run(Handle* h, const rafeast_params& prm, const double* Qd
   h->prof[7] = a.sl;
   // a graph of `steps` steps, replayed until done; the ring grows before a
   // replay that needs more slots, or is folded into D when it may not
-  const int steps = lz_replay_steps(h, tight);
+  const int steps = room.steps;
   std::vector<cudaEvent_t> evs;
   if (prof) {
     evs.resize(2 * steps + 1);
@@ -1449,12 +1529,7 @@ static void filter_lz_run(Handle* h, const rafeast_params& prm, const double* Qd
   std::vector<float> tk;  // per step: product ms, update ms (profiling)
   CocgCtl ctl;
   memset(&ctl, 0, sizeof(ctl));
-  if (!h->mem_total) {
-    size_t mem_free = 0;
-    RF_CUDA(cudaMemGetInfo(&mem_free, &h->mem_total));
-  }
-  const size_t budget = tight ? 0 : h->mem_total / LZ_RING_SHARE;
-  int k0 = 0, cap = (int)h->lz_slabs.size() * a.sl;
+  int k0 = 0, cap = P.cap;
   bool wrapped = false;
   const int max_replays = (prm.max_inner + 2) / steps + 2;
   if (fixed) {  // step 0 by FP64 sums: u_0 has no fixed-point copy; its w^T w gives u_1's unit
@@ -1481,11 +1556,10 @@ static void filter_lz_run(Handle* h, const rafeast_params& prm, const double* Qd
   for (int r = 0; r < max_replays && !ctl.done; ++r) {
     const int k = ctl.iter;
     if (k - k0 + steps + 1 > cap && !wrapped) {
-      const int64_t want = (int64_t)k + steps + 1;
-      const int got = lz_grow(h, a.stride, a.sl, 0, want, budget);
+      const int got = lz_grow(h, a.stride, room, (int64_t)k + steps + 1);
       if (got != cap) {
         cap = got;
-        lz_ring_upload(h, a, st);
+        lz_ring_upload(h, a, cap, st);
       }
     }
     if (k - k0 + steps + 1 > cap) {
@@ -1851,26 +1925,16 @@ static void filter_lz_batched(std::vector<BatchItem*>& items, Handle* owner, cud
   bool all_vf = true;
   double cells = 0.0;
   int max_inner = 1;
+  LzRoom room = lz_room(owner, tight);  // (replays are as long as the first handle asks)
+  std::vector<std::unique_ptr<RingUse>> use;
   for (int t = 0; t < cnt; ++t) {
     Handle* h = items[t]->h;
-    // (replays are as long as the first handle asks)
-    const int chunk = h->opt_chunk;
-    h->opt_chunk = owner->opt_chunk;
-    try {
-      P[t] = lz_setup<T>(h, *items[t]->prm, h->Q, h->AQ, h->theta_d, h->theta, h->m0, h->ldq,
-                         ctl_d + t, prof, tight, false, bs);
-    } catch (...) {
-      h->opt_chunk = chunk;
-      throw;
-    }
-    h->opt_chunk = chunk;
+    use.emplace_back(new RingUse(h));
+    P[t] = lz_setup<T>(h, *items[t]->prm, h->Q, h->AQ, h->theta_d, h->theta, h->m0, h->ldq,
+                       ctl_d + t, prof, room, false, bs);
     all_vf = all_vf && P[t].a.lcolidx != nullptr;
     cells += (double)P[t].a.stride;
     max_inner = std::max(max_inner, items[t]->prm->max_inner);
-  }
-  if (!owner->mem_total) {
-    size_t mem_free = 0;
-    RF_CUDA(cudaMemGetInfo(&mem_free, &owner->mem_total));
   }
   LzGroupDev<T> gd;
   gd.args = (const LzArgs<T>*)(bb + o_args);
@@ -1953,7 +2017,7 @@ static void filter_lz_batched(std::vector<BatchItem*>& items, Handle* owner, cud
   prepare(shp.dl, shp.dc, 0);
   owner->prof[6] = shp.dl * 100 + shp.dc;
   owner->prof[7] = P[0].a.sl;
-  const int steps = lz_replay_steps(owner, tight);
+  const int steps = room.steps;
   std::vector<cudaEvent_t> evs;
   if (prof) {
     evs.resize(2 * steps + 1);
@@ -1990,7 +2054,7 @@ static void filter_lz_batched(std::vector<BatchItem*>& items, Handle* owner, cud
   for (auto& c : ctl) memset(&c, 0, sizeof(c));
   std::vector<int> k0(cnt, 0), cap(cnt);
   std::vector<char> wrapped(cnt, 0);
-  for (int t = 0; t < cnt; ++t) cap[t] = (int)items[t]->h->lz_slabs.size() * P[t].a.sl;
+  for (int t = 0; t < cnt; ++t) cap[t] = P[t].cap;
   std::vector<float> tk;
   bool all_done = false;
   const int max_replays = (max_inner + 2) / steps + 2;
@@ -2001,13 +2065,11 @@ static void filter_lz_batched(std::vector<BatchItem*>& items, Handle* owner, cud
       const int k = ctl[t].iter;
       if (k - k0[t] + steps + 1 > cap[t] && !wrapped[t]) {
         // a batch's rings share a quarter of the device's memory by size
-        h->mem_total = owner->mem_total;
-        const size_t budget =
-            tight ? 0 : (size_t)(owner->mem_total / 4 * ((double)P[t].a.stride / cells));
-        const int got = lz_grow(h, P[t].a.stride, P[t].a.sl, 0, (int64_t)k + steps + 1, budget);
+        room.share = (double)P[t].a.stride / cells / LZ_RINGS_SHARE;
+        const int got = lz_grow(h, P[t].a.stride, room, (int64_t)k + steps + 1);
         if (got != cap[t]) {
           cap[t] = got;
-          lz_ring_upload(h, P[t].a, bs);
+          lz_ring_upload(h, P[t].a, cap[t], bs);
         }
       }
       if (k - k0[t] + steps + 1 > cap[t]) {
@@ -2149,9 +2211,9 @@ static void ensure_subspace_bufs(Handle* h, int m0) {
     if (h->theta_d) cudaFree(h->theta_d);
     h->Q = h->AQ = h->theta_d = nullptr;
     h->m0 = 0;
-    RF_CUDA(cudaMalloc(&h->Q, sizeof(double) * h->n * ldq));
-    RF_CUDA(cudaMalloc(&h->AQ, sizeof(double) * h->n * ldq));
-    RF_CUDA(cudaMalloc(&h->theta_d, sizeof(double) * (m0 + 1)));
+    RF_CUDA(dev_malloc(h->device, &h->Q, sizeof(double) * h->n * ldq));
+    RF_CUDA(dev_malloc(h->device, &h->AQ, sizeof(double) * h->n * ldq));
+    RF_CUDA(dev_malloc(h->device, &h->theta_d, sizeof(double) * (m0 + 1)));
     RF_CUDA(cudaMemsetAsync(h->Q, 0, sizeof(double) * h->n * ldq, h->stream));
     RF_CUDA(cudaMemsetAsync(h->AQ, 0, sizeof(double) * h->n * ldq, h->stream));
     h->ldq = ldq;
@@ -2437,6 +2499,7 @@ int rafeast_create(rafeast_t* out, int64_t n, int64_t nnz, const int32_t* row_pt
     RF_CUDA(cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking));
     RF_CUDA(cudaEventCreateWithFlags(&h->ev_in, cudaEventDisableTiming));
     RF_CUDA(cudaEventCreateWithFlags(&h->ev_out, cudaEventDisableTiming));
+    RF_CUDA(cudaEventCreateWithFlags(&h->lz_done, cudaEventDisableTiming));
     CallScope scope(h);
     // host copies for validation and reordering
     std::vector<int32_t> rp(n + 1), ci(nnz);
@@ -2543,8 +2606,8 @@ int rafeast_create(rafeast_t* out, int64_t n, int64_t nnz, const int32_t* row_pt
           va2[rp2[r] + t] = row[t].second;
         }
       }
-      RF_CUDA(cudaMalloc(&h->perm, sizeof(int32_t) * n));
-      RF_CUDA(cudaMalloc(&h->iperm, sizeof(int32_t) * n));
+      RF_CUDA(dev_malloc(h->device, &h->perm, sizeof(int32_t) * n));
+      RF_CUDA(dev_malloc(h->device, &h->iperm, sizeof(int32_t) * n));
       RF_CUDA(cudaMemcpy(h->perm, perm.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice));
       RF_CUDA(cudaMemcpy(h->iperm, ip.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice));
     }
@@ -2586,8 +2649,8 @@ int rafeast_create(rafeast_t* out, int64_t n, int64_t nnz, const int32_t* row_pt
       }
       if (twice) h->max_deg = 0;
       h->nnz_off = (int64_t)lci.size();
-      RF_CUDA(cudaMalloc(&h->lrowptr, sizeof(int32_t) * (n + 1)));
-      RF_CUDA(cudaMalloc(&h->lcolidx, sizeof(int32_t) * std::max<int64_t>(h->nnz_off, 1)));
+      RF_CUDA(dev_malloc(h->device, &h->lrowptr, sizeof(int32_t) * (n + 1)));
+      RF_CUDA(dev_malloc(h->device, &h->lcolidx, sizeof(int32_t) * std::max<int64_t>(h->nnz_off, 1)));
       RF_CUDA(cudaMemcpy(h->lrowptr, lrp.data(), sizeof(int32_t) * (n + 1),
                          cudaMemcpyHostToDevice));
       if (h->nnz_off)
@@ -2605,11 +2668,11 @@ int rafeast_create(rafeast_t* out, int64_t n, int64_t nnz, const int32_t* row_pt
         h->tile_max_union = t.max_union;
         h->tile_max_rows = t.max_rows;
         h->tile_ratio = (double)t.ucol.size() / (double)n;
-        RF_CUDA(cudaMalloc(&h->trow, sizeof(int32_t) * t.trow.size()));
-        RF_CUDA(cudaMalloc(&h->uoff, sizeof(int32_t) * t.uoff.size()));
-        RF_CUDA(cudaMalloc(&h->ucol, sizeof(int32_t) * t.ucol.size()));
-        RF_CUDA(cudaMalloc(&h->uself, sizeof(int32_t) * us.size()));
-        RF_CUDA(cudaMalloc(&h->lidx, sizeof(uint16_t) * lx.size()));
+        RF_CUDA(dev_malloc(h->device, &h->trow, sizeof(int32_t) * t.trow.size()));
+        RF_CUDA(dev_malloc(h->device, &h->uoff, sizeof(int32_t) * t.uoff.size()));
+        RF_CUDA(dev_malloc(h->device, &h->ucol, sizeof(int32_t) * t.ucol.size()));
+        RF_CUDA(dev_malloc(h->device, &h->uself, sizeof(int32_t) * us.size()));
+        RF_CUDA(dev_malloc(h->device, &h->lidx, sizeof(uint16_t) * lx.size()));
         RF_CUDA(cudaMemcpy(h->trow, t.trow.data(), sizeof(int32_t) * t.trow.size(),
                            cudaMemcpyHostToDevice));
         RF_CUDA(cudaMemcpy(h->uoff, t.uoff.data(), sizeof(int32_t) * t.uoff.size(),
@@ -2631,7 +2694,7 @@ int rafeast_create(rafeast_t* out, int64_t n, int64_t nnz, const int32_t* row_pt
             lrp[r + 1] = (int32_t)lci.size();
           }
           tile_local_index(n, lrp.data(), lci.data(), t, llx, us);
-          RF_CUDA(cudaMalloc(&h->llidx, sizeof(uint16_t) * llx.size()));
+          RF_CUDA(dev_malloc(h->device, &h->llidx, sizeof(uint16_t) * llx.size()));
           RF_CUDA(cudaMemcpy(h->llidx, llx.data(), sizeof(uint16_t) * llx.size(),
                              cudaMemcpyHostToDevice));
         }
@@ -2639,10 +2702,10 @@ int rafeast_create(rafeast_t* out, int64_t n, int64_t nnz, const int32_t* row_pt
     }
     std::vector<float> v32(nnz);
     for (int64_t k = 0; k < nnz; ++k) v32[k] = (float)va2[k];
-    RF_CUDA(cudaMalloc(&h->rowptr, sizeof(int32_t) * (n + 1)));
-    RF_CUDA(cudaMalloc(&h->colidx, sizeof(int32_t) * std::max<int64_t>(nnz, 1)));
-    RF_CUDA(cudaMalloc(&h->val64, sizeof(double) * std::max<int64_t>(nnz, 1)));
-    RF_CUDA(cudaMalloc(&h->val32, sizeof(float) * std::max<int64_t>(nnz, 1)));
+    RF_CUDA(dev_malloc(h->device, &h->rowptr, sizeof(int32_t) * (n + 1)));
+    RF_CUDA(dev_malloc(h->device, &h->colidx, sizeof(int32_t) * std::max<int64_t>(nnz, 1)));
+    RF_CUDA(dev_malloc(h->device, &h->val64, sizeof(double) * std::max<int64_t>(nnz, 1)));
+    RF_CUDA(dev_malloc(h->device, &h->val32, sizeof(float) * std::max<int64_t>(nnz, 1)));
     RF_CUDA(cudaMemcpy(h->rowptr, rp2.data(), sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice));
     if (nnz) {
       RF_CUDA(cudaMemcpy(h->colidx, ci2.data(), sizeof(int32_t) * nnz, cudaMemcpyHostToDevice));
@@ -2676,6 +2739,7 @@ void rafeast_destroy(rafeast_t hh) {
     if (p) cudaFree(p);
   if (h->ev_in) cudaEventDestroy(h->ev_in);
   if (h->ev_out) cudaEventDestroy(h->ev_out);
+  if (h->lz_done) cudaEventDestroy(h->lz_done);
   if (h->stream) cudaStreamDestroy(h->stream);
   delete h;
 }

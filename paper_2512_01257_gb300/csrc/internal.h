@@ -163,7 +163,7 @@ template <typename T> struct CocgArgs {
 
 // ---- real Lanczos form of the multi-shift solve (lanczos.cuh) ----------------
 constexpr int LZ_RUNS = 0x7fffffff;  // kstop of a column or node still iterating
-constexpr int LZ_SL = 32;            // most ring slots per slab
+constexpr int LZ_SL = 32;            // ring slots of a slab of up to a gigabyte
 constexpr int LZ_SLABS = 128;        // most slabs of a ring
 struct LzCol {  // per column
   double rr, irr;  // u_k^T u_k and its reciprocal
@@ -287,7 +287,6 @@ struct DevBuf {
 struct Handle {
   int device = 0;
   int num_sms = 0;
-  size_t mem_total = 0;  // bytes of device memory
   int64_t n = 0, nnz = 0;
   cudaStream_t user_stream = nullptr;
   cudaStream_t stream = nullptr;  // internal, non-blocking
@@ -362,11 +361,13 @@ struct Handle {
   std::vector<float> last_tk;        // dot, update kernel milliseconds per step
   // scratch, grown on demand and kept
   std::vector<DevBuf> bufs;
-  // slabs of the Lanczos ring (lanczos.cuh), kept for the next solve while
-  // their slots have this many bytes
+  // the Lanczos ring (lanczos.cuh): slabs of lz_slab_bytes each, kept for the next
+  // solve; lz_done is recorded behind the last filter that used them. All three
+  // under the rings' mutex (api.cu) but while lz_busy.
   std::vector<void*> lz_slabs;
-  int64_t lz_stride = 0;
-  int lz_sl = 0;
+  size_t lz_slab_bytes = 0;
+  bool lz_busy = false;
+  cudaEvent_t lz_done = nullptr;
   // launch accounting of the current call
   int launches = 0;
   int spmm_launches = 0;
