@@ -215,7 +215,8 @@ int rafeast_create(rafeast_t* out, int64_t n, int64_t nnz,
  * recurrence, a ring of Lanczos vectors (RAFEAST_OPT_UPDATE 0) for its next call.
  * A ring takes the chunk of RAFEAST_OPT_CHUNK + 2 vectors that a replay needs;
  * beyond that it grows with the steps of a filter to at most a sixteenth of the
- * device's memory, all rings on a device together to a quarter. When an allocation of the library fails, or
+ * device's memory, all rings on a device together to a quarter, and only while a
+ * sixteenth of the device stays free. When an allocation of the library fails, or
  * a ring may not grow otherwise, rings of handles that are not in a filter are
  * taken back first, the longest unused before the others; a filter that still
  * runs out of memory is run once more with the smallest ring. */

@@ -1122,10 +1122,12 @@ struct LzProblem {
 // ---- the ring of Lanczos vectors (Handle::lz_slabs) ---------------------------
 // Slots are allocated as a solve needs them. Beyond the slots a replay cannot do
 // without, a ring grows to a share of the device's memory (LZ_RING_SHARE), all
-// rings on the device together to a quarter of it; a solve with more steps than
-// slots folds full rings into its directions.
+// rings on the device together to a quarter of it, and a sixteenth of the device
+// stays free for what the solve and the program allocate next; a solve with
+// more steps than slots folds full rings into its directions.
 constexpr size_t LZ_RING_SHARE = 16;   // one ring: a sixteenth of the device's memory
 constexpr size_t LZ_RINGS_SHARE = 4;   // all rings
+constexpr size_t LZ_FREE_SHARE = 16;   // left free by growth
 constexpr int LZ_MAX_SL = 4096;        // slots of a slab made for larger ones
 static void lz_free(Handle* h) {
   lz_ring_drop(h);
@@ -1174,7 +1176,8 @@ static int lz_grow(Handle* h, int64_t stride, const LzRoom& room, int64_t want) 
       size_t mem_free = 0, total = 0;
       RF_CUDA(cudaMemGetInfo(&mem_free, &total));
       if ((double)(h->lz_slabs.size() + 1) * bytes > room.share * total) break;
-      if (ring_bytes(h->device) + bytes > total / LZ_RINGS_SHARE) {
+      if (ring_bytes(h->device) + bytes > total / LZ_RINGS_SHARE ||
+          mem_free < bytes + total / LZ_FREE_SHARE) {
         if (!ring_reclaim_locked(h->device)) break;
         continue;
       }

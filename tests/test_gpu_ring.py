@@ -54,6 +54,18 @@ def cube(lib):
         lib.rafeast_destroy(h)
 
 
+def test_ring_leaves_memory_to_others(lib, cube):
+    """With 6 GiB free a ring that took all it could use would leave a few hundred
+    megabytes; one that keeps a sixteenth of the device free takes the gibibyte
+    that it cannot do without, of about 1.6 with the filter's blocks."""
+    _, run = cube
+    hold = _hold_all_but(6 * GIB)
+    run(0)
+    left = _free()
+    del hold
+    assert left >= 4 * GIB
+
+
 def test_idle_rings_are_given_to_another_handle(lib, cube):
     """The second handle's blocks and smallest ring (0.6 GiB) do not fit the 0.35
     that are free: the first handle's idle ring makes room, and comes back for the
