@@ -1159,13 +1159,15 @@ static int lz_slab_slots(const Handle* h, int64_t stride) {
 }
 // slots of `stride` bytes: the least a replay needs, or it throws, and `want` of
 // them as far as there is room; returns the slots there are. A slab holds 32
-// slots of up to 32 MB, is a gigabyte while that is 8 slots, and 8 slots above.
+// slots of up to 32 MB, is a gigabyte while that is 8 slots, and 8 slots above:
+// the size grows with the slot's, so that a handle whose calls alternate between
+// widths keeps the slabs of the widest.
 static int lz_grow(Handle* h, int64_t stride, const LzRoom& room, int64_t want) {
   const int64_t per = room.per_slab(), gb = (int64_t)1 << 30;
   int64_t slab = stride * per;
   if (slab > gb) slab = std::max(gb, stride * std::min<int64_t>(per, 8));
   std::lock_guard<std::mutex> lock(g_ring_mu);
-  if ((int64_t)h->lz_slab_bytes != slab) ring_drop_locked(h);
+  if ((int64_t)h->lz_slab_bytes < slab) ring_drop_locked(h);
   if (h->lz_slabs.empty()) h->lz_slab_bytes = (size_t)slab;
   const size_t bytes = h->lz_slab_bytes;
   const int64_t sl = lz_slab_slots(h, stride), least = room.least();

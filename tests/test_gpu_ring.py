@@ -85,3 +85,14 @@ def test_idle_rings_are_given_to_another_handle(lib, cube):
     assert float((first - again).norm(dim=1).max()) <= bound
 
 
+def test_alternating_widths_keep_the_ring(lib, cube):
+    """A narrow filter takes the slabs of a wide one: the free memory stays as it is
+    from the second call on (workspaces grow with the widest)."""
+    _, run = cube
+    left = []
+    for m0 in (24, 96, 24, 96, 24):
+        run(0, m0, 40)
+        left.append(_free())
+    assert len(set(left[1:])) == 1
+
+
