@@ -2144,6 +2144,8 @@ static void filter_lz_batched(std::vector<BatchItem*>& items, Handle* owner, cud
       if (ctl[t].done) lz_collapse<T>(h, P[t].a, k0[t], ctl[t].iter, true, h->stream);
       lz_finish_filter<T>(h, P[t], h->Q, h->ldq, items[t]->Qt, ctl[t], items[t]->fs, h->stream);
     } catch (const Err& e) {
+      // (memory: the batch runs once more with the smallest rings)
+      if (e.code == RAFEAST_ERR_OUT_OF_MEMORY && !tight) throw;
       items[t]->err = e.code;
     }
   }
