@@ -144,6 +144,21 @@ extern "C" {
                                      * (default) every update complete (the    *
                                      * deferred form moves more bytes and      *
                                      * measured slower)                        */
+#define RAFEAST_OPT_RING_SLOTS 18   /* most Lanczos vectors (slots of n rows)  *
+                                     * that a filter keeps before it folds     *
+                                     * them into its quadrature sum: 0         *
+                                     * (default) as memory allows, or 4 to     *
+                                     * 2^20. Setting it gives the handle's     *
+                                     * ring back to the device; see Memory     *
+                                     * below                                   */
+#define RAFEAST_OPT_RING_SLOTS 18   /* most Lanczos vectors (slots of n rows)  *
+                                     * that a filter keeps before it folds     *
+                                     * them into its quadrature sum: 0         *
+                                     * (default) as memory allows, or 4 to     *
+                                     * 2^20. Batched solves follow the first   *
+                                     * handle's setting. Setting it gives the  *
+                                     * handle's ring back to the device; see   *
+                                     * Memory below                            */
 #define RAFEAST_OPT_TEST_STALL 9    /* test hook: bytes (multiple of 16) that  *
                                      * every bulk-copy stage waits for and no *
                                      * copy delivers, so the bounded wait     *

@@ -1149,7 +1149,7 @@ struct LzRoom {
 static LzRoom lz_room(const Handle* h, bool tight) {
   LzRoom r;
   r.tight = tight;
-  r.limit = tight ? 4 : 0;
+  r.limit = tight ? 4 : h->opt_ring;
   r.steps = std::min(62, std::max(2, h->opt_chunk + (h->opt_chunk & 1)));
   if (r.limit) r.steps = std::min(r.steps, std::max(2, (r.limit - 2) & ~1));
   return r;
@@ -2801,6 +2801,11 @@ int rafeast_set_option(rafeast_t hh, int key, int64_t value) {
     case RAFEAST_OPT_DEFER:
       if (value < 0 || value > 1) return RAFEAST_ERR_INVALID_ARG;
       h->opt_defer = (int)value;
+      return RAFEAST_OK;
+    case RAFEAST_OPT_RING_SLOTS:
+      if (value != 0 && (value < 4 || value > (1 << 20))) return RAFEAST_ERR_INVALID_ARG;
+      h->opt_ring = (int)value;
+      lz_ring_drop(h);
       return RAFEAST_OK;
     case RAFEAST_OPT_DENSE:
       if (value < 0 || value > 1) return RAFEAST_ERR_INVALID_ARG;

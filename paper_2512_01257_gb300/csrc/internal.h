@@ -368,6 +368,7 @@ struct Handle {
   size_t lz_slab_bytes = 0;
   bool lz_busy = false;
   cudaEvent_t lz_done = nullptr;
+  int opt_ring = 0;  // most slots of the ring (0: as memory allows)
   // launch accounting of the current call
   int launches = 0;
   int spmm_launches = 0;

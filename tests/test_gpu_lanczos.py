@@ -1,11 +1,11 @@
 """Real Lanczos form of the multi-shift filter (the default route) against the
 oracle's conjugate orthogonal CG after a fixed number of steps.
 
-The ring of the Lanczos vectors is taken up in chunks of 32 steps (or of the
-step cap plus one when that is smaller), so the step counts lie at the edges of
-a chunk; the widths leave ragged 16-byte chunks of columns and ragged column
-blocks; the node counts reach each instance of the pass over the ring (1, 2,
-4, 8 and two passes). solve_tol = 0: every system runs to the cap.
+The ring holds every step here, so one pass over it ends the filter (rings that
+are folded: test_gpu_ring.py). The step counts lie at the edges of 32 steps, the
+slots of a slab and the rows of the collapse's tiles; the widths leave ragged
+16-byte chunks of columns and ragged column blocks; the node counts fill one to
+twelve lanes of the warp that has a column's nodes. solve_tol = 0: every system runs to the cap.
 
 Tolerance (backward errors): a step rounds each value a few times (2^2), which
 is an error of the matrix of at most 2^2 eps ||A|| per step; k <= 70 steps make
