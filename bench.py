@@ -938,10 +938,8 @@ def main():
                                  "ms_per_launch": prof[f"{other}_ms"] / max(prof[f"{other}_launches"], 1)},
                 "share_of_step": (prof["update_ms"] + prof["dots_ms"]) / ms}
 
-    # (unit-weight Laplacians of eight or more neighbours a row: neighbour sums
-    # in 64-bit integers, which the FP64 pipe does not bind)
-    vf, nnz_off = _unit_laplacian(lap)
-    if prec == R.RAFEAST_FP64 and pre == "dots" and not (vf and nnz_off >= 8 * lap.n):
+    # (neighbour sums in 64-bit integers: the FP64 pipe does not bind them)
+    if prec == R.RAFEAST_FP64 and pre == "dots" and not prof["fixed_sums"]:
         roofline = _fp64_dots_roofline(roofline, prof, lap, dev)
     # the sparse product the metric names: w = L u over the CSR pattern (tiled:
     # the gathered rows staged in shared memory) with the step's dot products

@@ -266,8 +266,11 @@ int rafeast_set_option(rafeast_t h, int key, int64_t value);
  * launches, milliseconds, bytes; update-kernel launches, milliseconds, bytes;
  * the kernel shapes of the last multi-shift solve as 10000*c + 100*lanes +
  * chunks per lane, c the CTAs per SM the chosen kernel instance is compiled
- * for (0: the default instance; dot kernel, update kernel; chosen by the
- * autotuner). Bytes count A once (nnz*(4+s) + 4(n+1), s = 4 or 8) plus each state
+ * for (0: the default instance), 100000 more when the product's neighbour sums
+ * were formed in 64-bit integers, 1000000 + 100*(chunks per block) + c for a
+ * tiled product; then the update kernel's, which is 0 for the real Lanczos
+ * recurrence (its update has one shape). The autotuner chooses the shapes.
+ * Bytes count A once (nnz*(4+s) + 4(n+1), s = 4 or 8) plus each state
  * column the launch reads or writes once: the product reads u_k and writes
  * L u_k, the update reads both and u_{k-1} and writes u_{k+1} (complex COCG
  * forms: the dot kernel reads r, the update kernel reads and writes r and p

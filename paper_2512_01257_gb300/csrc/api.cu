@@ -1493,8 +1493,9 @@ static void filter_lz_run(Handle* h, const rafeast_params& prm, const double* Qd
     cb = h->opt_tile_cb;  // forced block width (tests)
     occ = 0;
   }
-  h->prof[6] = cb ? 1000000 + cb * 100 + occ : occ * 10000 + a.lanes * 100 + a.cpl;
-  h->prof[7] = a.sl;
+  h->prof[6] = cb ? 1000000 + cb * 100 + occ
+                  : (fixed ? 100000 : 0) + occ * 10000 + a.lanes * 100 + a.cpl;
+  h->prof[7] = 0;
   // a graph of `steps` steps, replayed until done; the ring grows before a
   // replay that needs more slots, or is folded into D when it may not
   const int steps = room.steps;
@@ -2021,7 +2022,7 @@ static void filter_lz_batched(std::vector<BatchItem*>& items, Handle* owner, cud
   }
   prepare(shp.dl, shp.dc, 0);
   owner->prof[6] = shp.dl * 100 + shp.dc;
-  owner->prof[7] = P[0].a.sl;
+  owner->prof[7] = 0;
   const int steps = room.steps;
   std::vector<cudaEvent_t> evs;
   if (prof) {

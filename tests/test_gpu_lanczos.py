@@ -354,3 +354,37 @@ def test_fixed_point_sums_are_as_accurate_as_fp64_sums(lib):
     finally:
         lib.rafeast_destroy(h)
     assert np.exp(np.mean(np.log(err[0] / err[1]))) <= np.sqrt(2.0)
+
+
+@pytest.mark.parametrize("kind,fixed", [("knn", True), ("rgg", True), ("complete", True), ("hub", False),
+                                        (500, True), (636, True), (660, False), ("grid", False)])
+def test_which_neighbour_sums_run(lib, kind, fixed):
+    """Fixed point for eight or more neighbours a row and n max deg / mean deg <=
+    41,000 (a number: that many vertices of a star and circulant, 25,000, 40,500
+    and 43,700), never for read values, in float or in a filter of another form."""
+    import torch
+    lap = G.grid2d(20, 23, shift=0.3) if kind == "grid" else \
+        _star_and_circulant(kind) if isinstance(kind, int) else _dense_graph(kind)
+    h = lib.rafeast_create(lap.row_ptr, lap.col_idx, lap.values, lap.shift)
+    try:
+        for prec, values_free, update, exp in ((lib.RAFEAST_FP64, 0, 0, fixed), (lib.RAFEAST_FP64, 1, 0, False),
+                                               (lib.RAFEAST_MIXED, 0, 0, False), (lib.RAFEAST_FP64, 0, 2, False)):
+            lib.rafeast_set_option(h, lib.RAFEAST_OPT_VALUES_FREE, values_free)
+            lib.rafeast_set_option(h, lib.RAFEAST_OPT_UPDATE, update)
+            prm = lib.make_params(0.31, 4.0, 6, 2, 1.0, 1e-2, 1e-10, 1, 20, prec, lib.RAFEAST_FORM_DIRECT)
+            Q = colmajor_dev(OF.random_start(lap.n, 6, 1))
+            lib.rafeast_filter(h, prm, Q, None, torch.zeros_like(Q))
+            p = lib.rafeast_profile(h, reset=False)
+            assert p["fixed_sums"] is exp and (update or p["update_shape"] == 0), (prec, values_free, update)
+    finally:
+        lib.rafeast_destroy(h)
+
+
+@pytest.mark.parametrize("m0,nc", [(6, 2), (69, 4)])
+@pytest.mark.parametrize("n", [500, 636])
+def test_fixed_point_sums_with_a_hub_against_dense(lib, monkeypatch, n, m0, nc):
+    """test_fixed_point_sums_against_dense on graphs with one vertex joined to all
+    that take the fixed-point route (its own is over the rule's line)."""
+    import test_gpu_lanczos as here
+    monkeypatch.setattr(here, "_dense_graph", lambda kind: _star_and_circulant(n))
+    here.test_fixed_point_sums_against_dense(lib, "star", m0, nc)
