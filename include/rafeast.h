@@ -117,17 +117,21 @@ extern "C" {
                                      * its off-diagonal pattern alone, with   *
                                      * L r = deg r - sum of neighbours; 1:    *
                                      * always read the values                 */
-#define RAFEAST_OPT_TILED 14        /* seed dot kernel of the multi-shift    *
-                                     * float32 solve with the streamed update: *
-                                     * 0 (default) tiled (row tiles whose      *
-                                     * gathered rows are staged in shared      *
-                                     * memory) when the matrix has tiles, the  *
-                                     * autotuner choosing between it and the   *
-                                     * register gathers; 1 register gathers    *
-                                     * only; 2 tiled only (when it has tiles)  */
-#define RAFEAST_OPT_TILE_CB 15      /* with RAFEAST_OPT_TILED = 2: column     *
-                                     * pairs per block of the tiled dot kernel *
-                                     * (4 or 8; 0 = autotuned)                 */
+#define RAFEAST_OPT_TILED 14        /* sparse product of the multi-shift     *
+                                     * float32 solve (real Lanczos, or COCG    *
+                                     * with the streamed update): 0 (default)  *
+                                     * tiled (row tiles whose gathered rows    *
+                                     * are staged in shared memory) when the   *
+                                     * matrix has tiles, the autotuner         *
+                                     * choosing between it and the register    *
+                                     * gathers; 1 register gathers only; 2     *
+                                     * tiled only (when it has tiles)          */
+#define RAFEAST_OPT_TILE_CB 15      /* with RAFEAST_OPT_TILED = 2: chunks of a  *
+                                     * row per block of the tiled product (4   *
+                                     * real columns each in the real Lanczos   *
+                                     * recurrence: 4, 5, 8 or 10; 2 complex in *
+                                     * the COCG forms: 4 or 8; 0 and others =  *
+                                     * autotuned)                              */
 #define RAFEAST_OPT_DENSE 16        /* FP64 Gram matrices (Cholesky-QR,       *
                                      * Rayleigh-Ritz, rafeast_gram): 0 (default)*
                                      * on the tensor cores, FP64 values split   *

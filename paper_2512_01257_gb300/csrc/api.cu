@@ -1054,7 +1054,7 @@ static void filter_ms_dev(Handle* h, const rafeast_params& prm, const double* Qd
     shp.dt = dot_cb;
     h->tuned.push_back(std::make_pair(key, shp));
   }
-  if (can_tile && h->opt_tiled == 2 && h->opt_tile_cb > 0) {
+  if (can_tile && h->opt_tiled == 2 && (h->opt_tile_cb == 4 || h->opt_tile_cb == 8)) {
     dot_cb = h->opt_tile_cb;  // forced block width (tests)
     dot_occ = 0;
   }
@@ -2813,7 +2813,8 @@ int rafeast_set_option(rafeast_t hh, int key, int64_t value) {
       h->opt_dense = (int)value;
       return RAFEAST_OK;
     case RAFEAST_OPT_TILE_CB:
-      if (value != 0 && value != 4 && value != 8) return RAFEAST_ERR_INVALID_ARG;
+      if (value != 0 && value != 4 && value != 5 && value != 8 && value != 10)
+        return RAFEAST_ERR_INVALID_ARG;
       h->opt_tile_cb = (int)value;
       return RAFEAST_OK;
     case RAFEAST_OPT_CPL:

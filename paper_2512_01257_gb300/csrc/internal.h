@@ -333,8 +333,8 @@ struct Handle {
   int opt_solver = 1;  // 0: COCG per shift, 1: multi-shift COCG (default)
   int opt_update = 0;  // multi-shift update: 0 auto, 1 gathered products, 2 streamed
   int opt_values_free = 0;  // 0: values-free gathers for unit Laplacians, 1: never
-  int opt_tiled = 0;        // seed dot kernel: 0 auto (tiled when built), 1 never, 2 only tiled
-  int opt_tile_cb = 0;      // tiled dot kernel: forced column pairs per block (0: autotuned)
+  int opt_tiled = 0;        // float product: 0 auto (tiled when built), 1 never, 2 only tiled
+  int opt_tile_cb = 0;      // tiled product: forced 16-byte chunks per block (0: autotuned)
   int opt_dense = 0;        // FP64 Gram matrices: 0 tensor cores (digit split), 1 FP64 pipe
   int opt_defer = 0;        // 1: deferred shifted updates with the tiled dot kernel, 0: never
   // quadrature nodes [shard_j0, shard_j1) of the N_c this filter sums over
