@@ -1175,9 +1175,9 @@ static int lz_grow(Handle* h, int64_t stride, const LzRoom& room, int64_t want) 
   want = std::max(want, least);
   while ((int64_t)h->lz_slabs.size() * sl < want && h->lz_slabs.size() < (size_t)LZ_SLABS) {
     if ((int64_t)h->lz_slabs.size() * sl >= least) {
+      if ((double)(h->lz_slabs.size() + 1) * bytes > room.share * h->mem_total) break;
       size_t mem_free = 0, total = 0;
       RF_CUDA(cudaMemGetInfo(&mem_free, &total));
-      if ((double)(h->lz_slabs.size() + 1) * bytes > room.share * total) break;
       if (ring_bytes(h->device) + bytes > total / LZ_RINGS_SHARE ||
           mem_free < bytes + total / LZ_FREE_SHARE) {
         if (!ring_reclaim_locked(h->device)) break;
@@ -2500,6 +2500,8 @@ int rafeast_create(rafeast_t* out, int64_t n, int64_t nnz, const int32_t* row_pt
   try {
     RF_CUDA(cudaGetDevice(&h->device));
     RF_CUDA(cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device));
+    size_t mem_free = 0;
+    RF_CUDA(cudaMemGetInfo(&mem_free, &h->mem_total));
     h->n = n;
     h->nnz = nnz;
     h->shift = diag_shift;

@@ -287,6 +287,7 @@ struct DevBuf {
 struct Handle {
   int device = 0;
   int num_sms = 0;
+  size_t mem_total = 0;  // bytes of device memory
   int64_t n = 0, nnz = 0;
   cudaStream_t user_stream = nullptr;
   cudaStream_t stream = nullptr;  // internal, non-blocking

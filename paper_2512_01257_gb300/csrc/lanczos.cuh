@@ -164,6 +164,13 @@ __device__ void lz_column_scalars(const LzArgs<T>& a, int k, int c0, int c1, con
       st.irr = irr;
       st.bad = !unit || !isfinite(rr) || !isfinite(ul) || !isfinite((double)cf.alpha) ||
                !isfinite((double)cf.g) || !isfinite((double)cf.s) || (rr > 0.0 && !(cf.s > (T)0));
+      // the column stops at this step, broken down or converged (an eigenvector's
+      // last scale can leave the range): its next vector is 0, for an infinite one
+      // would meet a coefficient of 0 in the sum over the ring
+      if (st.bad) {
+        cf.alpha = cf.g = cf.s = (T)0;
+        E = 0;
+      }
     }
     a.cf[c] = cf;
     if constexpr (NS == 3) a.qe[c] = E;
@@ -663,9 +670,9 @@ __device__ __forceinline__ void lz_comp_col(const LzArgs<T>& a, const LzRing& ri
 // D += sum_k c_k u_k over the steps [k0, k1), rows [r0, r1): the pass that ends
 // a solve whose steps all fit the ring. A thread takes RPT rows of one chunk of
 // columns, UB slots' loads in flight together; the coefficients come through
-// L1 (one 16-byte read per RPT rows). Bound by HBM: each u read once. What a
-// stopped column leaves in later slots (infinite or NaN where its last scale
-// left the range) is not read into D, whatever its neighbours in the chunk do.
+// L1 (one 16-byte read per RPT rows). Bound by HBM: each u read once. Slots past
+// a column's stop are read with a coefficient of 0 while its neighbours in the
+// chunk go on; lz_column_scalars keeps them finite.
 // ---------------------------------------------------------------------------
 template <typename T>
 __device__ __forceinline__ void lz_sum_rows(const LzArgs<T>& a, const LzRing& ring, int cap, int k0,
@@ -675,12 +682,9 @@ __device__ __forceinline__ void lz_sum_rows(const LzArgs<T>& a, const LzRing& ri
   const int nq = a.nq, per = THREADS / nq;
   const int q = threadIdx.x % nq, rs = threadIdx.x / nq;
   if (rs >= per) return;
-  int kq = k0, ks[V];  // the chunk of columns has coefficients below kq, column v below ks[v]
+  int kq = k0;  // the chunk of columns has coefficients below kq
 #pragma unroll
-  for (int v = 0; v < V; ++v) {
-    ks[v] = a.col[q * V + v].kstop;
-    kq = max(kq, min(k1, ks[v]));
-  }
+  for (int v = 0; v < V; ++v) kq = max(kq, min(k1, a.col[q * V + v].kstop));
   for (int64_t r = r0 + rs; r < r1; r += (int64_t)RPT * per) {
     int64_t o[RPT];
     T d[RPT][V];
@@ -710,8 +714,7 @@ __device__ __forceinline__ void lz_sum_rows(const LzArgs<T>& a, const LzRing& ri
             T uv[V];
             lz_get(uq[y][x], uv);
 #pragma unroll
-            for (int v = 0; v < V; ++v)
-              if (k + y < ks[v]) d[x][v] = fma(c[v], uv[v], d[x][v]);
+            for (int v = 0; v < V; ++v) d[x][v] = fma(c[v], uv[v], d[x][v]);
           }
         }
     }
@@ -736,11 +739,10 @@ __device__ __forceinline__ void lz_apply_rows(const LzArgs<T>& a, const LzRing& 
   const int nq = a.nq, nc = a.nc, per = THREADS / nq;
   const int q = threadIdx.x % nq, rs = threadIdx.x / nq;
   if (rs >= per) return;
-  int kq = k0, fl = 0, ks[V];
+  int kq = k0, fl = 0;
 #pragma unroll
   for (int v = 0; v < V; ++v) {
-    ks[v] = a.col[q * V + v].kstop;
-    kq = max(kq, min(k1, ks[v]));
+    kq = max(kq, min(k1, a.col[q * V + v].kstop));
 #pragma unroll
     for (int j = 0; j < JB; ++j)
       if (j0 + j < nc) fl |= a.pflag[(int64_t)(q * V + v) * nc + j0 + j] << (2 * j);
@@ -796,12 +798,7 @@ __device__ __forceinline__ void lz_apply_rows(const LzArgs<T>& a, const LzRing& 
         if (k + y < kq) {
           T uv[RPT][V];
 #pragma unroll
-          for (int x = 0; x < RPT; ++x) {
-            lz_get(uq[y][x], uv[x]);
-#pragma unroll
-            for (int v = 0; v < V; ++v)  // (as in lz_sum_rows)
-              if (k + y >= ks[v]) uv[x][v] = (T)0;
-          }
+          for (int x = 0; x < RPT; ++x) lz_get(uq[y][x], uv[x]);
           if (j0 == 0) {
             T c[V];
             lz_get(__ldg(reinterpret_cast<const Q*>(a.cc + (int64_t)(k + y - k0) * a.ld + q * V)), c);
