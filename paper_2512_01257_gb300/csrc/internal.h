@@ -382,7 +382,7 @@ void* scratch(Handle* h, int slot, size_t bytes);  // keep-alive buffer per slot
 void ensure_dyn_smem(const void* fn, size_t bytes);
 enum Slot {
   S_STATE = 0, S_DACC, S_QT, S_TMP1, S_TMP2, S_SCAL, S_GRAM, S_SMALL, S_OMEGA,
-  S_AQ2, S_IO1, S_IO2, S_BATCH, S_TPART, S_SHARD, S_LZ, S_LZP, S_LZC, S_LZQ, S_COUNT
+  S_AQ2, S_IO1, S_IO2, S_BATCH, S_TPART, S_SHARD, S_LZP, S_LZC, S_LZQ, S_COUNT
 };
 
 // ---- host math (hostmath.cpp) ------------------------------------------------

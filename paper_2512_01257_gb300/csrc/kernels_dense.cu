@@ -563,7 +563,8 @@ void tall_gemm(const double* X, int64_t n, int m, int ldx, const double* M, int 
 // One SM issues 2 FP64 lane operations a clock, so the m^3 / 6 products of the
 // factorisation alone take 22 us at m = 80; the inverse, as many again, is
 // spread over the chip, where a column costs a latency chain of m steps. (Both
-// in one CTA, the inverse one column per thread: 234 us; now 55 us.)
+// in one CTA, the inverse one column per thread: 441 us in the launch list of the
+// kNN solve, 80 and 100 columns; now 170 and 29 us.)
 // ---------------------------------------------------------------------------
 // a / b from the rounded reciprocal ib: one step on the residual rounds the product
 // as the quotient (P. Markstein, IBM J. Res. Develop. 34, 1990); a ib alone has a
