@@ -667,7 +667,9 @@ void launch_spmm_real(int64_t n, const int32_t* rp, const int32_t* ci, const T* 
   const int mc = (k + 1) / 2;
   // eight lanes (128 bytes of a row) and the fewest column blocks of at most 4
   // chunks a lane. With the layout moves: 200,000 x 80 889 -> 871 us, 2,000 x 24
-  // 30.2 -> 24.4 us.
+  // 30.2 -> 24.4 us. Narrower blocks leave lanes idle and are still ahead of four
+  // lanes of the wide instance: one column of 200,000 rows 407 -> 147 us in FP64,
+  // 94 -> 72 us in float.
   const int G = 8, blocks = (mc + 4 * G - 1) / (4 * G), cpl = (mc + G * blocks - 1) / (G * blocks);
   if (cpl == 1)
     spmm_inst<T, 1, 6>(n, rp, ci, val, mc, ld, (T)sL, (T)sI, X, Y, G, cpl, blocks, num_sms, s);
